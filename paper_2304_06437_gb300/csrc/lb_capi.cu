@@ -47,17 +47,35 @@ size_t storage_bytes(int s) {
   }
 }
 
-// Build a 4-D TMA descriptor (x, y, z, direction) of the population array;
-// box = one plane of one brick for all directions.
-int make_tensor_map(lb_ctx* ctx) {
+PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
   static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
   if (!encode) {
     cudaDriverEntryPointQueryResult q;
     void* fn = nullptr;
     cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q);
-    if (e != cudaSuccess || q != cudaDriverEntryPointSuccess || !fn) return LB_E_CUDA;
+    if (e != cudaSuccess || q != cudaDriverEntryPointSuccess || !fn) return nullptr;
     encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
   }
+  return encode;
+}
+
+// A 4-D TMA descriptor (x, y, z, field) of nf fields of g.vol elements at
+// base; box = one plane of bx x by nodes for all fields.
+bool encode_map(const Geometry& g, CUtensorMap* map, CUtensorMapDataType dt, size_t es, void* base, int nf, int bx,
+                int by) {
+  auto encode = tensor_map_encoder();
+  if (!encode) return false;
+  cuuint64_t dims[4] = {cuuint64_t(g.nx), cuuint64_t(g.ny), cuuint64_t(g.nz), cuuint64_t(nf)};
+  cuuint64_t strides[3] = {cuuint64_t(g.pitch) * es, cuuint64_t(g.pitch) * g.ny * es, cuuint64_t(g.vol) * es};
+  cuuint32_t box[4] = {cuuint32_t(bx), cuuint32_t(by), 1u, cuuint32_t(nf)};
+  cuuint32_t estr[4] = {1, 1, 1, 1};
+  return encode(map, dt, 4, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// The descriptor of the population array: box = one plane of one brick for
+// all directions.
+int make_tensor_map(lb_ctx* ctx) {
   CUtensorMapDataType dt;
   switch (ctx->storage) {
     case LB_F64: dt = CU_TENSOR_MAP_DATA_TYPE_FLOAT64; break;
@@ -65,17 +83,12 @@ int make_tensor_map(lb_ctx* ctx) {
     case LB_F16S: dt = CU_TENSOR_MAP_DATA_TYPE_FLOAT16; break;
     default: dt = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16; break;
   }
-  const Geometry& g = ctx->g;
-  const cuuint64_t es = ctx->elem_bytes;
-  cuuint64_t dims[4] = {cuuint64_t(g.nx), cuuint64_t(g.ny), cuuint64_t(g.nz), cuuint64_t(g.q)};
-  cuuint64_t strides[3] = {cuuint64_t(g.pitch) * es, cuuint64_t(g.pitch) * g.ny * es, cuuint64_t(g.vol) * es};
-  cuuint32_t box[4] = {cuuint32_t(ctx->plan.bx), cuuint32_t(ctx->plan.by), 1u, cuuint32_t(g.q)};
-  cuuint32_t estr[4] = {1, 1, 1, 1};
-  CUresult r = encode(&ctx->tmap, dt, 4, ctx->f, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                      CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? LB_OK : LB_E_CUDA;
+  return encode_map(ctx->g, &ctx->tmap, dt, ctx->elem_bytes, ctx->f, ctx->g.q, ctx->plan.bx, ctx->plan.by)
+             ? LB_OK
+             : LB_E_CUDA;
 }
+
+size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
 
 // Host moment fields cross to and from the device through a buffer of at
 // most this size, in two halves: while the context stream converts the chunk
@@ -178,6 +191,12 @@ void drop_step_graph(lb_ctx* ctx) {
   ctx->step_graph = nullptr;
 }
 
+bool make_field_map(lb_ctx* ctx, CUtensorMap* map, void* base, int nf, int bx, int by) {
+  return encode_map(ctx->g, map,
+                    ctx->real_bytes == 8 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
+                    ctx->real_bytes, base, nf, bx, by);
+}
+
 int ctx_replan(lb_ctx* ctx, const void* variant, int bz) {
   if (!ctx || ctx->scheme != LB_SCHEME_FUSED) return LB_E_INVAL;
   FusedPlan p;
@@ -186,6 +205,7 @@ int ctx_replan(lb_ctx* ctx, const void* variant, int bz) {
   LB_TRY_CUDA(cudaStreamSynchronize(ctx->stream));
   // a captured step pair holds the old shell buffers and brick plan
   drop_step_graph(ctx);
+  drop_moment_run(ctx);
   const size_t aux_bytes = size_t(2) * size_t(p.parity_elems) * ctx->real_bytes;
   void* aux = nullptr;
   LB_TRY_CUDA(cudaMalloc(&aux, aux_bytes));
@@ -197,9 +217,11 @@ int ctx_replan(lb_ctx* ctx, const void* variant, int bz) {
   const FusedPlan old_plan = ctx->plan;
   void* old_aux = ctx->aux;
   const size_t old_bytes = ctx->aux_bytes;
+  const bool old_own = ctx->own_aux;
   ctx->plan = p;
   ctx->aux = aux;
   ctx->aux_bytes = aux_bytes;
+  ctx->own_aux = true;
   int rc = make_tensor_map(ctx);
   if (rc == LB_OK) rc = cuda_status(k1_configure(ctx));
   if (rc == LB_OK) rc = after_state_change(ctx);  // rebuild the shell from the populations
@@ -208,11 +230,12 @@ int ctx_replan(lb_ctx* ctx, const void* variant, int bz) {
     ctx->plan = old_plan;
     ctx->aux = old_aux;
     ctx->aux_bytes = old_bytes;
+    ctx->own_aux = old_own;
     make_tensor_map(ctx);
     cudaFree(aux);
     return rc;
   }
-  cudaFree(old_aux);
+  if (old_own) cudaFree(old_aux);
   return LB_OK;
 }
 
@@ -433,11 +456,23 @@ int lb_create(int32_t lattice, const int64_t dims[3], double tau, const lb_bound
       ctx->aux_bytes = k0_aux_bytes(g, ctx->storage);
     }
     ctx->f_bytes = size_t(q) * size_t(g.vol) * ctx->elem_bytes;
-    cudaError_t e = cudaMalloc(&ctx->f, ctx->f_bytes);
+    // one allocation: the populations, then the shells or moment arrays; runs
+    // in moment form use both (the shells are rebuilt at their end)
+    const size_t aux_at = align256(ctx->f_bytes);
+    size_t want = aux_at + ctx->aux_bytes;
+    const size_t least = want;
+    if (ctx->scheme == LB_SCHEME_FUSED && !g.zlink[0] && !g.zlink[1])
+      want = std::max(want, moment_scratch_elems(g, ctx->storage) * ctx->real_bytes);
+    cudaError_t e = cudaMalloc(&ctx->f, want);
+    if (e == cudaErrorMemoryAllocation && want > least) {
+      cudaGetLastError();
+      want = least;
+      e = cudaMalloc(&ctx->f, want);
+    }
     if (e != cudaSuccess) { rc = cuda_status(e); break; }
+    ctx->f_alloc = want;
     if (ctx->aux_bytes) {
-      e = cudaMalloc(&ctx->aux, ctx->aux_bytes);
-      if (e != cudaSuccess) { rc = cuda_status(e); break; }
+      ctx->aux = static_cast<char*>(ctx->f) + aux_at;
       e = cudaMemsetAsync(ctx->aux, 0, ctx->aux_bytes, ctx->stream);
       if (e != cudaSuccess) { rc = cuda_status(e); break; }
     }
@@ -477,8 +512,9 @@ void lb_destroy(lb_ctx* ctx) {
   DeviceGuard guard(ctx->device);
   if (ctx->stream) cudaStreamSynchronize(ctx->stream);
   drop_step_graph(ctx);
+  drop_moment_run(ctx);
   if (ctx->f) cudaFree(ctx->f);
-  if (ctx->aux) cudaFree(ctx->aux);
+  if (ctx->aux && ctx->own_aux) cudaFree(ctx->aux);
   if (ctx->d_status) cudaFree(ctx->d_status);
   if (ctx->d_red) cudaFree(ctx->d_red);
   if (ctx->d_uprev) cudaFree(ctx->d_uprev);
@@ -653,6 +689,11 @@ int lb_step(lb_ctx* ctx, int64_t n) {
   if (n > 1 && (ctx->g.zlink[0] || ctx->g.zlink[1])) return LB_E_INVAL;
   DeviceGuard guard(ctx->device);
   int64_t i = 0;
+  if (n >= kMomentMinSteps && moment_plan(ctx)) {
+    const cudaError_t e = moment_run(ctx, n);
+    if (e == cudaSuccess) ctx->steps_done += n;
+    return cuda_status(e);
+  }
   // long runs of the fused scheme replay a captured pair of steps: one graph
   // launch per two steps instead of two launches, each with its host-side
   // argument set-up (what dominates the step of a small domain)

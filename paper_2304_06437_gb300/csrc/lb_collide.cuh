@@ -314,14 +314,33 @@ LB_DEV R post(const Coef<R>& k) {
   else return fma_r(w, even, wodd);
 }
 
-// full regularized collision of one node: ft -> ft*; the two members of a
-// velocity pair share the even part and take -/+ the odd part
-template <class L, class R, bool FORCE>
-LB_DEV void collide(const R (&f)[L::Q], const Phys<R>& ph, R (&out)[L::Q]) {
-  Mom<R> m;
-  moments<L, R, FORCE>(f, ph, m);
-  Coef<R> k;
-  coeffs<L, R, FORCE>(m, ph, k);
+// the state of a node in moment form: the number of coefficients of its
+// post-collision set, and their list, f(i, ref) for i = 0 .. n_coef - 1 in the
+// order of the coefficient fields (lb_k3.cuh)
+template <class L>
+LB_HD constexpr int n_coef() { return L::D == 2 ? 6 : 10; }
+template <class L, class R, class F>
+LB_DEV void each_coef(Coef<R>& k, F&& f) {
+  if constexpr (L::D == 2) {
+    // the internal y axis carries no velocities in 2D
+    f(std::integral_constant<int, 0>{}, k.A);
+    f(std::integral_constant<int, 1>{}, k.B[0]);
+    f(std::integral_constant<int, 2>{}, k.B[2]);
+    f(std::integral_constant<int, 3>{}, k.C[0]);
+    f(std::integral_constant<int, 4>{}, k.C[2]);
+    f(std::integral_constant<int, 5>{}, k.C2[od(0, 2)]);
+  } else {
+    f(std::integral_constant<int, 0>{}, k.A);
+    static_for<0, 3>([&](auto I) { f(std::integral_constant<int, 1 + decltype(I)::value>{}, k.B[decltype(I)::value]); });
+    static_for<0, 3>([&](auto I) { f(std::integral_constant<int, 4 + decltype(I)::value>{}, k.C[decltype(I)::value]); });
+    static_for<0, 3>([&](auto I) { f(std::integral_constant<int, 7 + decltype(I)::value>{}, k.C2[decltype(I)::value]); });
+  }
+}
+
+// the post-collision set of a node from its coefficients; the two members of
+// a velocity pair share the even part and take -/+ the odd part
+template <class L, class R>
+LB_DEV void post_all(const Coef<R>& k, R (&out)[L::Q]) {
   static_assert(L::cx(0) == 0 && L::cy(0) == 0 && L::cz(0) == 0, "direction 0 is the rest population");
   out[0] = post<L, R, 0>(k);
   static_for<0, n_pairs<L>()>([&](auto P) {
@@ -334,6 +353,16 @@ LB_DEV void collide(const R (&f)[L::Q], const Phys<R>& ph, R (&out)[L::Q]) {
     out[a] = fma_r(w, even, wodd);
     out[b] = fma_r(w, even, -wodd);
   });
+}
+
+// full regularized collision of one node: ft -> ft*
+template <class L, class R, bool FORCE>
+LB_DEV void collide(const R (&f)[L::Q], const Phys<R>& ph, R (&out)[L::Q]) {
+  Mom<R> m;
+  moments<L, R, FORCE>(f, ph, m);
+  Coef<R> k;
+  coeffs<L, R, FORCE>(m, ph, k);
+  post_all<L, R>(k, out);
 }
 
 }  // namespace lbgb

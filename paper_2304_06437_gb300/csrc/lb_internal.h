@@ -44,7 +44,23 @@ struct FusedPlan {
   size_t smem_bytes;
 };
 
-struct Status;
+struct K3Variant;
+struct LeaveVariant;
+
+// Runs of several steps in moment form (lb_k3.cuh): the compiled tile and
+// ending brick launches of a context, its TMA descriptors (coefficient sets A
+// and B by tile, set A by brick) and the recorded steps.
+struct MomentRun {
+  int state = 0;  // 0 not planned yet, 1 usable, -1 not available to this context
+  const K3Variant* v = nullptr;
+  const LeaveVariant* lv = nullptr;
+  int bz = 0;
+  CUtensorMap tmap_a, tmap_b, tmap_leave;
+  cudaGraphExec_t graph = nullptr;
+};
+constexpr int kMomentGraphSteps = 8;
+// shortest lb_step() call that runs in moment form
+constexpr int64_t kMomentMinSteps = 4;
 
 }  // namespace lbgb
 
@@ -63,8 +79,13 @@ struct lb_ctx {
   size_t real_bytes;      // arithmetic element size (shells, moments)
   void* f;                // the population array: q * vol elements
   size_t f_bytes;
+  // f's allocation continues past the populations: the shells (fused
+  // scheme) follow them, and where two sets of coefficient fields (lb_k3.cuh)
+  // need more, the allocation is that much longer
+  size_t f_alloc;
   void* aux;              // shells (fused) or moment arrays (two-pass)
   size_t aux_bytes;
+  bool own_aux;           // aux is an allocation of its own (else part of f's)
   lbgb::FusedPlan plan;
   int parity;             // shell parity holding the current post-collision halo
   CUtensorMap tmap;       // TMA descriptor of the population array (fused)
@@ -78,6 +99,7 @@ struct lb_ctx {
   // the brick plan or the shell buffers change)
   cudaGraphExec_t step_graph = nullptr;
   int graph_parity = 0;
+  lbgb::MomentRun mr;
 };
 
 namespace lbgb {
@@ -104,6 +126,19 @@ void drop_step_graph(lb_ctx* ctx);
 cudaError_t k1_step(lb_ctx* ctx);
 cudaError_t k1_bootstrap(lb_ctx* ctx);  // fill the current shell parity from f
 cudaError_t k1_configure(lb_ctx* ctx);  // one-time kernel attributes
+
+// ---- runs of several steps in moment form (lb_k3_plan.cu)
+// arithmetic-type elements that the two coefficient sets span from f on (0:
+// no compiled tile for this lattice and storage)
+size_t moment_scratch_elems(const Geometry& g, int storage);
+// whether the context can run in moment form; plans it on the first call
+bool moment_plan(lb_ctx* ctx);
+// n >= 2 steps of a planned context
+cudaError_t moment_run(lb_ctx* ctx, int64_t n);
+void drop_moment_run(lb_ctx* ctx);
+// TMA descriptor of nf fields of the arithmetic type at base, boxes of bx x by
+// x 1 x nf (lb_capi.cu)
+bool make_field_map(lb_ctx* ctx, CUtensorMap* map, void* base, int nf, int bx, int by);
 
 // ---- state conversion, readout and reductions (lb_aux.cu)
 cudaError_t aux_set_populations(lb_ctx* ctx, const double* f_dev);

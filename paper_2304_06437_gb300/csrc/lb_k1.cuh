@@ -283,21 +283,12 @@ __device__ __forceinline__ void export_face(const Coef<R>& kc, ShellSpot<R> s) {
   });
 }
 
-// Collide the completed (rounded) state of one node once more and export the
-// populations that leave the brick through the flagged faces.
-template <class L, class S, class R, bool FORCE, bool LINK = false>
-__device__ __forceinline__ void export_node(const K1Args<R>& args, const R (&fin)[L::Q], int x, int y, int zd,
+// Export the populations of one node (its post-collision coefficients kc) that
+// leave the brick through the flagged faces.
+template <class L, class R, bool LINK>
+__device__ __forceinline__ void export_coef(const K1Args<R>& args, const Coef<R>& kc, int x, int y, int zd,
                                             unsigned faces, int bI, int bJ, int bK) {
   constexpr int NXF = count_dirs<L>(0, 1), NYF = count_dirs<L>(1, 1), NZF = count_dirs<L>(2, 1);
-  R fr[L::Q];
-  static_for<0, L::Q>([&](auto A_) {
-    constexpr int a = decltype(A_)::value;
-    fr[a] = round_to_storage<S, R>(fin[a]);
-  });
-  Mom<R> m;
-  moments<L, R, FORCE>(fr, args.ph, m);
-  Coef<R> kc;
-  coeffs<L, R, FORCE>(m, args.ph, kc);
   R* shn = args.sh_next;
   // LINK: the shell of a slab context, with ghost planes / brick rows
   const int zg = LINK ? args.zg : 0;
@@ -331,6 +322,23 @@ __device__ __forceinline__ void export_node(const K1Args<R>& args, const R (&fin
       export_face<L, R, 2, 1>(
           kc, {shn + args.sz_off + ((int64_t(LINK ? args.nbzs : args.nbz) + bK + zg) * NZF) * nyx + row, nyx});
   }
+}
+
+// Collide the completed (rounded) state of one node once more and export the
+// populations that leave the brick through the flagged faces.
+template <class L, class S, class R, bool FORCE, bool LINK = false>
+__device__ __forceinline__ void export_node(const K1Args<R>& args, const R (&fin)[L::Q], int x, int y, int zd,
+                                            unsigned faces, int bI, int bJ, int bK) {
+  R fr[L::Q];
+  static_for<0, L::Q>([&](auto A_) {
+    constexpr int a = decltype(A_)::value;
+    fr[a] = round_to_storage<S, R>(fin[a]);
+  });
+  Mom<R> m;
+  moments<L, R, FORCE>(fr, args.ph, m);
+  Coef<R> kc;
+  coeffs<L, R, FORCE>(m, args.ph, kc);
+  export_coef<L, R, LINK>(args, kc, x, y, zd, faces, bI, bJ, bK);
 }
 
 // Export entry e of a brick shape: its face (0 W, 1 E, 2 S, 3 N) and the
@@ -381,8 +389,12 @@ __device__ __forceinline__ void export_one_face(const Phys<R>& ph, const R (&fin
 // PHPLANE: the arguments sit in shared memory (batched sweeps); the collision
 // then reads its physical constants as one block copy at the start of each
 // use (loads issued ahead of the collision, not one per operand inside it).
+//
+// INC: the last step of a run in moment form (lb_k3.cuh): the array holds the
+// nodes' post-collision coefficients in its first n_coef fields (type R; the
+// TMA descriptor names those), and the populations are written over them.
 template <class L, class S, class R, int BX, int BY, int NS, int WB, int NXW, bool FORCE, int TS = 0,
-          bool LINK = false, int MINB = 1, bool PHPLANE = false>
+          bool LINK = false, int MINB = 1, bool PHPLANE = false, bool INC = false>
 __device__ __forceinline__ bool k1_brick(const CUtensorMap* tmap_p, const K1Args<R>& args, const int bI,
                                          const int bJ, const int bK) {
   using Sh = K1Shape<L, S, R, BX, BY, NS, WB, NXW, TS, MINB>;
@@ -395,6 +407,10 @@ __device__ __forceinline__ bool k1_brick(const CUtensorMap* tmap_p, const K1Args
   constexpr int PMAX = Sh::PMAX, NEXW = Sh::NEXW, QP = Sh::QP, VEC = Sh::VEC, PE = Sh::PE;
   constexpr int WY = Sh::WY;
   constexpr int WSTRIDE = int(align128(Sh::WIN) / sizeof(R));  // between window buffers
+  constexpr int NC = n_coef<L>();
+  // bytes one plane's load brings: all populations, or (INC) the coefficients
+  constexpr size_t LOAD = INC ? size_t(NC) * BY * BX * sizeof(R) : Sh::SLOT;
+  static_assert(LOAD <= Sh::SLOT, "a plane of coefficients fits a slot");
   using Vec = typename std::conditional<sizeof(R) == 4, float4, double2>::type;
 
   extern __shared__ __align__(128) unsigned char smem[];
@@ -482,7 +498,7 @@ __device__ __forceinline__ bool k1_brick(const CUtensorMap* tmap_p, const K1Args
     for (int s = 0; s < NS; ++s) {
       const int zz = z0 + s;
       if (zz < z1) {
-        mbar_arrive_expect_tx(&bars[s], static_cast<uint32_t>(Sh::SLOT));
+        mbar_arrive_expect_tx(&bars[s], static_cast<uint32_t>(LOAD));
         tma_load_4d(slots + size_t(s) * Q * BY * BX, tmap_p, x0, y0, zz, 0, &bars[s]);
         ++issued;
       }
@@ -670,13 +686,21 @@ __device__ __forceinline__ bool k1_brick(const CUtensorMap* tmap_p, const K1Args
       if constexpr (PHPLANE) phl = args.ph;  // loads in flight during the wait
       if (!mbar_wait_bounded(&bars[slot], (k / NS) & 1, kWaitLimitNs)) return false;
       if (active) {
-        const S* sl = slots + size_t(slot) * Q * BY * BX + ty * BX + tx;
-        R fl[Q], own[Q];
-        static_for<0, Q>([&](auto A_) {
-          constexpr int a = decltype(A_)::value;
-          fl[a] = load_as<S, R>(sl[a * BY * BX]);
-        });
-        collide<L, R, FORCE>(fl, PHPLANE ? phl : args.ph, own);
+        R own[Q];
+        if constexpr (INC) {
+          const R* sl = reinterpret_cast<const R*>(slots + size_t(slot) * Q * BY * BX) + ty * BX + tx;
+          Coef<R> kc;
+          each_coef<L, R>(kc, [&](auto I, R& v) { v = sl[decltype(I)::value * BY * BX]; });
+          post_all<L, R>(kc, own);
+        } else {
+          const S* sl = slots + size_t(slot) * Q * BY * BX + ty * BX + tx;
+          R fl[Q];
+          static_for<0, Q>([&](auto A_) {
+            constexpr int a = decltype(A_)::value;
+            fl[a] = load_as<S, R>(sl[a * BY * BX]);
+          });
+          collide<L, R, FORCE>(fl, PHPLANE ? phl : args.ph, own);
+        }
         static_for<0, Q>([&](auto A_) {
           constexpr int a = decltype(A_)::value;
           if constexpr (is_lateral<L>(a)) win[lat_index<L>(a) * WPLANE + wbase] = own[a];
@@ -942,7 +966,7 @@ __device__ __forceinline__ bool k1_brick(const CUtensorMap* tmap_p, const K1Args
       // refill the slot consumed by plane c with plane c + NS
       if (tid == 0 && c >= z0 && c < z1 && c + NS < z1) {
         const int slot = (c - z0) % NS;
-        mbar_arrive_expect_tx(&bars[slot], static_cast<uint32_t>(Sh::SLOT));
+        mbar_arrive_expect_tx(&bars[slot], static_cast<uint32_t>(LOAD));
         tma_load_4d(slots + size_t(slot) * Q * BY * BX, tmap_p, x0, y0, c + NS, 0, &bars[slot]);
         ++issued;
       }
@@ -990,6 +1014,17 @@ __global__ void __launch_bounds__(K1Shape<L, S, R, BX, BY, NS, WB, NXW, TS, MINB
   const int b = blockIdx.x;
   k1_brick<L, S, R, BX, BY, NS, WB, NXW, FORCE, TS, LINK, MINB>(&tmap, args, b % nbx, (b / nbx) % nby,
                                                                 b / (nbx * nby));
+}
+
+// The last step of a run in moment form: coefficients -> populations, one CTA
+// per brick column of the domain's own plan, in place.
+template <class L, class S, class R, int BX, int BY, int NS, bool FORCE>
+__global__ void __launch_bounds__(K1Shape<L, S, R, BX, BY, NS, 2, 0>::NT, 1)
+    k1_leave_step(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ K1Args<R> args) {
+  const int nbx = args.nbx, nby = args.nby;
+  const int b = blockIdx.x;
+  k1_brick<L, S, R, BX, BY, NS, 2, 0, FORCE, 0, false, 1, false, true>(&tmap, args, b % nbx, (b / nbx) % nby,
+                                                                       b / (nbx * nby));
 }
 
 // One launch per time step of many domains (a batch): a persistent grid whose
@@ -1043,7 +1078,8 @@ __global__ void __launch_bounds__(K1Shape<L, S, R, BX, BY, NS, WB, NXW, TS, MINB
 // Shell bootstrap: collide every brick-boundary node of the current state and
 // export its outgoing populations into shell parity `sh_next` (used once after
 // the state is set from outside; the steps keep the shell current).
-template <class L, class S, class R, int BX, int BY, bool FORCE>
+// INC: from the coefficient fields of a run in moment form, before its last step.
+template <class L, class S, class R, int BX, int BY, bool FORCE, bool INC = false>
 __global__ void __launch_bounds__(256) k1_bootstrap(const __grid_constant__ K1Args<R> args) {
   constexpr int Q = L::Q;
   const int64_t n = int64_t(args.nx) * args.ny * args.nz;
@@ -1062,15 +1098,22 @@ __global__ void __launch_bounds__(256) k1_bootstrap(const __grid_constant__ K1Ar
     const bool eU = z == z1 - 1 && (z1 < args.nz || args.per[2] || args.zlink[1]);
     if (!(eW || eE || eS || eN || eD || eU)) continue;
     const int64_t o = x + args.pitch * (y + int64_t(args.ny) * z);
-    const S* fg = static_cast<const S*>(args.f);
-    R fr[Q];
-    static_for<0, Q>([&](auto A_) {
-      constexpr int a = decltype(A_)::value;
-      fr[a] = load_as<S, R>(fg[a * args.vol + o]);
-    });
     const unsigned faces = (eW ? kFaceW : 0u) | (eE ? kFaceE : 0u) | (eS ? kFaceS : 0u) | (eN ? kFaceN : 0u) |
                            (eD ? kFaceD : 0u) | (eU ? kFaceU : 0u);
-    export_node<L, S, R, FORCE, true>(args, fr, x, y, z, faces, bI, bJ, bK);
+    if constexpr (INC) {
+      const R* cg = static_cast<const R*>(args.f);
+      Coef<R> kc;
+      each_coef<L, R>(kc, [&](auto I, R& v) { v = cg[decltype(I)::value * args.vol + o]; });
+      export_coef<L, R, true>(args, kc, x, y, z, faces, bI, bJ, bK);
+    } else {
+      const S* fg = static_cast<const S*>(args.f);
+      R fr[Q];
+      static_for<0, Q>([&](auto A_) {
+        constexpr int a = decltype(A_)::value;
+        fr[a] = load_as<S, R>(fg[a * args.vol + o]);
+      });
+      export_node<L, S, R, FORCE, true>(args, fr, x, y, z, faces, bI, bJ, bK);
+    }
   }
 }
 
