@@ -77,6 +77,9 @@ struct Phys {
   R cs2;     // 1/3 rounded to R
   // products of the constants above, formed once in FP64 on the host
   R c15rho0, c15om1, c3rho0, c45rho0, c45om1, c9rho0, c9om1, c3g, c9g;
+  // negated constants, for packed arithmetic (lb_pair.cuh), whose operands
+  // carry no sign
+  R n_rho0, n_inv_rho0, n_cs2, n15rho0, n15om1, n3g;
 };
 
 LB_DEV float fma_r(float a, float b, float c) { return fmaf(a, b, c); }

@@ -48,14 +48,14 @@ struct K3Variant;
 struct LeaveVariant;
 
 // Runs of several steps in moment form (lb_k3.cuh): the compiled tile and
-// ending brick launches of a context, its TMA descriptors (coefficient sets A
-// and B by tile, set A by brick) and the recorded steps.
+// ending brick launches of a context, its TMA descriptors and the recorded steps.
 struct MomentRun {
   int state = 0;  // 0 not planned yet, 1 usable, -1 not available to this context
   const K3Variant* v = nullptr;
   const LeaveVariant* lv = nullptr;
   int bz = 0;
-  CUtensorMap tmap_a, tmap_b, tmap_leave;
+  CUtensorMap maps[2];  // sets A and B, boxes of a tile
+  CUtensorMap tmap_leave;
   cudaGraphExec_t graph = nullptr;
 };
 constexpr int kMomentGraphSteps = 8;
@@ -128,9 +128,19 @@ cudaError_t k1_bootstrap(lb_ctx* ctx);  // fill the current shell parity from f
 cudaError_t k1_configure(lb_ctx* ctx);  // one-time kernel attributes
 
 // ---- runs of several steps in moment form (lb_k3_plan.cu)
-// arithmetic-type elements that the two coefficient sets span from f on (0:
-// no compiled tile for this lattice and storage)
+// arithmetic-type elements that the two coefficient sets and their edge
+// records span from f on (0: no compiled tile for this lattice and storage)
 size_t moment_scratch_elems(const Geometry& g, int storage);
+// where the edge records begin: past both sets and past the populations (which
+// the conversion to set A or B still reads)
+inline int64_t moment_edge_at(const Geometry& g) {
+  const int sets = g.d == 2 ? 12 : 20;
+  return int64_t(g.q > sets ? g.q : sets) * g.vol;
+}
+// elements of one set's edge records for tiles bx wide
+inline int64_t moment_edge_elems(const Geometry& g, int bx) {
+  return (int64_t(2) * ((g.nx + bx - 1) / bx) * g.ny * g.nz * (g.d == 2 ? 6 : 10) + 31) / 32 * 32;
+}
 // whether the context can run in moment form; plans it on the first call
 bool moment_plan(lb_ctx* ctx);
 // n >= 2 steps of a planned context

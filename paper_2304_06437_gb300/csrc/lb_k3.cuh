@@ -20,37 +20,61 @@
 // (D3Q27 FP32) or by instruction issue close to it (D3Q19 FP32); the moment
 // form moves 2 n_coef: 80 instead of 152 / 216 bytes per update for D3Q19 /
 // D3Q27 FP32.  It also needs no shell: source and destination differ, so a
-// tile reads its one-node halo straight from the source fields (L2 holds what
-// the neighbouring tiles read), and nothing is collided twice.
+// tile reads its one-node halo from the source set (L2 holds what the
+// neighbouring tiles read), and nothing is collided twice.  Measured per step
+// on one GB300, single-step launches against this form: D3Q19 FP32 512^3 35.2
+// -> 63.5 GLUPS (5.1 TB/s, 0.75 of the copy rate), 256^3 31.9 -> 60.3, 32^3
+// 24.8 -> 4.3 us; D3Q27 FP32 256^3 25.6 -> 47.0 (0.56); D3Q19 / D3Q27 FP64 96^3
+// 2.19 -> 3.17 / 1.10 -> 1.88 (bound by the FP64 rate).  What bounds the FP32
+// kernels: instruction issue (62 % of the slots) and, without the halo warps'
+// part, 71 GLUPS.
 //
 // Memory: the two sets of coefficient fields live in the population array
 // itself -- set A in fields 0 .. n_coef - 1, set B in the n_coef fields after
-// field q/2 -- which the allocation extends to 2 n_coef fields where q is
-// smaller (the shell buffers, idle meanwhile, are that extension in 3D).
+// it -- and its allocation goes on through the shell buffers (idle meanwhile,
+// rebuilt at the end), which hold what 2 n_coef fields exceed q by and the edge
+// records below.
 //
 // Layout of a launch: a CTA owns a tile of bx x by nodes and sweeps bz planes.
 // TMA streams the tile's coefficients plane by plane into a ring of shared
-// slots; each node thread evaluates its post-collision set and puts the
-// laterally moving populations into a shared window (three buffers); halo
-// warps do the same for the one-node ring around the tile, from loads issued
-// one plane ahead, and only for the populations that enter the tile.  One
-// split barrier per plane: a warp arrives once its part of a window is
-// written and waits when it needs the whole.
+// slots; each node thread evaluates the post-collision set of its node, or of
+// the two nodes x and x + 1 (NPT = 2: packed FP32x2 arithmetic, lb_pair.cuh),
+// and puts the laterally moving populations into a shared window (three
+// buffers).  Halo warps fill the one-node ring around the tile, from loads
+// issued a plane ahead: with the populations that enter from the neighbouring
+// tiles, or, where the tile borders an x or y wall, with the bounce-back
+// values of the wall's own nodes, so that the node warps gather without any
+// test for walls.  One split barrier per plane: a warp arrives once its part
+// of a window is written and waits when it needs the whole.
 #pragma once
 
 #include "lb_k1.cuh"
+#include "lb_pair.cuh"
 
 namespace lbgb {
 
-template <class R>
+// Edge records: the coefficients of the nodes in the first (side 0) and last
+// (side 1) column of every tile, NC consecutive values a node and consecutive
+// along y, which the neighbouring tiles' ring columns are read from.  (Read
+// from the fields, every value is a sector of its own; D3Q19 64 x 8 tiles with
+// little L1 cache beside their shared memory: 51.9 against 59.9 GLUPS.)
+// Record of row r = y + ny z of tile column tI.
+LB_HD inline int64_t k3_edge(int side, int tI, int ntx, int64_t rows, int64_t r) {
+  return (int64_t(side) * ntx + tI) * rows + r;
+}
+
+// V: the type of a thread's values, R or f32x2 (two nodes)
+template <class R, class V>
 struct K3Args {
-  Phys<R> ph;
+  Phys<V> ph;
   int nx, ny, nz;
   int64_t pitch, vol;
   int per[3];
   int bz, ntx, nty, ntz;  // sweep length, tiles along x and y, bricks along z
   const R* src;           // coefficient fields read, and
   R* dst;                 // written: field i at + i * vol
+  const R* esrc;          // edge records of the two sets (see k3_edge)
+  R* edst;
   int* status;
   uint32_t vol32;         // vol / 32 (rows are padded to 32 elements)
   R bb[27][8];
@@ -64,42 +88,90 @@ LB_HD constexpr int nonlateral_dir() {
   return -1;
 }
 
-template <class L, class R, int BX, int BY, int NS, int MINB>
+template <class L, class R, int BX, int BY, int NS, int NPT, int MINB>
 struct K3Shape {
+  using V = typename std::conditional<NPT == 2, f32x2, R>::type;
   static constexpr int Q = L::Q;
   static constexpr int NC = n_coef<L>();
-  static constexpr int NTM = BX * BY;  // threads that own a node
   static constexpr int NYF = count_dirs<L>(1, 1);
-  static constexpr int NLAT = n_lateral<L>();
   static constexpr int PY = NYF > 0 ? 1 : 0;
-  static constexpr int WX = BX + 2;
-  static constexpr int WY = BY + 2 * PY;
-  static constexpr int WPLANE = WX * WY;
-  // halo entries, one per thread of the halo warps: south and north rows
-  // (whole warps), then the west and east columns with the corners
-  static constexpr int HROW = NYF > 0 ? 2 * BX : 0;
-  static constexpr int HWARPS = (HROW + 2 * WY + 31) / 32;
+  static constexpr int HB = BX / NPT;      // node threads per row
+  static constexpr int NTM = HB * BY;      // node threads
+  static constexpr int WY = BY + 2 * PY;   // window rows
+  // Window of one direction: rows of the tile and its ring.  A direction with
+  // cx = 0 needs no ring along x: rows of BX values.  The others have rows of
+  // BX + 2, and with two nodes per thread the even and the odd nodes of a row
+  // apart (E(0) .. E(HB), then O(-1) .. O(HB - 1)), so that a thread's pair,
+  // shifted by one node, is two loads of consecutive lanes.
+  LB_HD static constexpr int row(int a) { return L::cx(a) == 0 ? BX : BX + 2; }
+  LB_HD static constexpr int off(int a) {
+    int n = 0;
+    for (int b = 0; b < a; ++b)
+      if (is_lateral<L>(b)) n += WY * row(b);
+    return n;
+  }
+  // position of the tile's column xl (-1 .. BX) in a row of a moving direction
+  LB_HD static constexpr int col(int xl) {
+    return NPT == 2 ? ((xl & 1) ? HB + 1 + (xl + 1) / 2 : xl / 2) : xl + 1;
+  }
+  // halo threads: south and north rows (one per node thread column), then the
+  // west and east columns with the corners, each column in warps of its own
+  // (a warp of two faces runs both in turn, and is then what the others wait for)
+  static constexpr int HROW = NYF > 0 ? 2 * HB : 0;
+  static constexpr int HCOL = NYF > 0 ? (WY + 31) / 32 * 32 : 16;
+  static constexpr int HWARPS = (HROW + 2 * HCOL) / 32;
   static constexpr int NT = NTM + 32 * HWARPS;
-  static constexpr size_t SLOT = size_t(NC) * BY * BX * sizeof(R);
-  static constexpr size_t WIN = align128(size_t(NLAT) * WPLANE * sizeof(R));
-  static constexpr size_t OFF_WIN = align128(NS * SLOT);
-  static constexpr size_t OFF_BAR = OFF_WIN + 3 * WIN;
-  static constexpr size_t SMEM = OFF_BAR + align128((NS + 3) * sizeof(uint64_t));
   static constexpr int NWARPS = NT / 32;
+  static constexpr int SLOTN = NC * BY * BX;  // elements of one plane of the tile
+  static constexpr size_t WIN = align128(size_t(off(Q)) * sizeof(R));
+  static constexpr size_t OFF_WIN = align128(size_t(NS) * SLOTN * sizeof(R));
   static constexpr size_t SMEM_CAP = (size_t(228) * 1024) / MINB - 1024;
+  static constexpr int NW = 3;  // window buffers
+  // the halo threads' coefficients, HD planes deep (rows: V, columns: R)
+  static constexpr int HD = 4;
+  static constexpr size_t HSTAGE = size_t(NC) * (HROW * sizeof(V) + 2 * HCOL * sizeof(R));
+  static constexpr size_t OFF_HALO = OFF_WIN + NW * WIN;
+  static constexpr size_t OFF_BAR = align128(OFF_HALO + HD * HSTAGE);
+  static constexpr size_t SMEM = OFF_BAR + align128((NS + NW) * sizeof(uint64_t));
   static_assert(SMEM <= SMEM_CAP, "shared memory of the shape exceeds its share of the SM");
   static_assert(NTM % 32 == 0 && NT <= 1024, "whole warps");
   static_assert(BY == 1 || NYF > 0, "a 2D tile has one internal row");
+  static_assert(NPT == 1 || (std::is_same<R, float>::value && BX % 2 == 0), "pairs are FP32");
+  static_assert(HROW % 32 == 0, "a halo warp holds rows or columns, not both");
 };
 
+// lane l of a thread's value
+template <class R>
+LB_DEV R& lane_of(R& v, int) { return v; }
+LB_DEV float& lane_of(f32x2& v, int l) { return l == 0 ? v.x : v.y; }
+
+// lane l's coefficients as one record (16- or 8-byte stores)
+template <class L, class R, class V>
+LB_DEV void put_record(Coef<V>& k, R* e, int l) {
+  using R2 = typename std::conditional<sizeof(R) == 4, float2, double2>::type;
+  R rec[n_coef<L>()];
+  each_coef<L, V>(k, [&](auto I, V& v) { rec[decltype(I)::value] = l == 0 ? lane_of(v, 0) : lane_of(v, 1); });
+#pragma unroll
+  for (int i = 0; i < n_coef<L>(); i += 2) reinterpret_cast<R2*>(e)[i / 2] = R2{rec[i], rec[i + 1]};
+}
+
+template <class S, class R>
+LB_DEV R round_value(R v) { return round_to_storage<S, R>(v); }
+template <class S>
+LB_DEV f32x2 round_value(f32x2 v) { return round_pair<S>(v); }
+
 // One step of one brick (tile column tI, tJ, sweep tK): src -> dst.
-template <class L, class S, class R, int BX, int BY, int NS, bool FORCE, int MINB>
-__device__ __forceinline__ void k3_brick(const CUtensorMap* tmap_p, const K3Args<R>& args, const int tI, const int tJ,
-                                         const int tK) {
-  using Sh = K3Shape<L, R, BX, BY, NS, MINB>;
-  constexpr int Q = L::Q, NC = Sh::NC, NTM = Sh::NTM, NYF = Sh::NYF, PY = Sh::PY;
-  constexpr int WX = Sh::WX, WY = Sh::WY, WPLANE = Sh::WPLANE, HROW = Sh::HROW;
+template <class L, class S, class R, int BX, int BY, int NS, int NPT, bool FORCE, int MINB>
+__device__ __forceinline__ void k3_brick(
+    const CUtensorMap* tmap_p, const K3Args<R, typename K3Shape<L, R, BX, BY, NS, NPT, MINB>::V>& args, const int tI,
+    const int tJ, const int tK) {
+  using Sh = K3Shape<L, R, BX, BY, NS, NPT, MINB>;
+  using V = typename Sh::V;
+  constexpr int Q = L::Q, NC = Sh::NC, NTM = Sh::NTM, NYF = Sh::NYF, PY = Sh::PY, HB = Sh::HB;
+  constexpr int WY = Sh::WY, HROW = Sh::HROW, NW = Sh::NW;
+  constexpr int RM = BX + 2;  // row of a moving direction
   constexpr int WSTRIDE = int(Sh::WIN / sizeof(R));
+  constexpr int SLOTN = Sh::SLOTN;
 
   extern __shared__ __align__(128) unsigned char smem[];
   R* slots = reinterpret_cast<R*>(smem);
@@ -122,16 +194,23 @@ __device__ __forceinline__ void k3_brick(const CUtensorMap* tmap_p, const K3Args
   const int ze = nbU ? z1 : z1 - 1;
   auto zwrap = [&](int z) { return z < 0 ? z + nz : (z >= nz ? z - nz : z); };
 
+  // faces of the tile at a wall
+  const bool wallW = x0 == 0 && !args.per[0], wallE = x0 + bxa == nx && !args.per[0];
+  const bool wallS = y0 == 0 && !args.per[1], wallN = y0 + bya == ny && !args.per[1];
+
   int issued = 0;  // planes whose load was issued (thread 0's count)
+  // thread 0: load plane zb + k into slot k % NS
+  auto load_plane = [&](int k) {
+    uint64_t* bar = &bars[k % NS];
+    mbar_arrive_expect_tx(bar, uint32_t(SLOTN * sizeof(R)));
+    tma_load_4d(slots + (k % NS) * SLOTN, tmap_p, x0, y0, zwrap(zb + k), 0, bar);
+    ++issued;
+  };
   if (tid == 0) {
     for (int s = 0; s < NS; ++s) mbar_init(&bars[s], 1);
-    for (int s = 0; s < 3; ++s) mbar_init(&wbars[s], Sh::NWARPS);
+    for (int s = 0; s < NW; ++s) mbar_init(&wbars[s], Sh::NWARPS);
     fence_barrier_init();
-    prefetch_tmap(tmap_p);
-    for (int s = 0; s < NS && zb + s <= ze; ++s, ++issued) {
-      mbar_arrive_expect_tx(&bars[s], static_cast<uint32_t>(Sh::SLOT));
-      tma_load_4d(slots + size_t(s) * NC * BY * BX, tmap_p, x0, y0, zwrap(zb + s), 0, &bars[s]);
-    }
+    for (int s = 0; s < NS && zb + s <= ze; ++s) load_plane(s);
   }
   __syncthreads();
 
@@ -139,149 +218,293 @@ __device__ __forceinline__ void k3_brick(const CUtensorMap* tmap_p, const K3Args
   // end (on undefined values, like the rest of the launch), so that every warp
   // still arrives at every barrier
   bool dead = false;
-  // windows: plane zb + k uses buffer k % 3.  A warp arrives when it has put its
-  // populations of a plane into the window and waits just before it gathers
-  // them, with the gather and collision of the plane before in between.  A
-  // warp that has passed plane k's barrier knows that every warp has gathered
-  // plane k - 2, so with three buffers it may fill plane k + 1's.
+  // windows: plane zb + k uses buffer k % NW.  A warp arrives when it has put
+  // its populations of a plane into the window and waits just before it
+  // gathers them, with the gather and collision of the plane before in between.
+  // A warp that has passed plane k's barrier knows that every warp has gathered
+  // plane k - 2, so it may fill the buffer of plane k + NW - 2.
   auto window_ready = [&](int k) {
     __syncwarp();
-    if (tid % 32 == 0) mbar_arrive(&wbars[k % 3]);
+    if (tid % 32 == 0) mbar_arrive(&wbars[k % NW]);
   };
   auto window_wait = [&](int k) {
-    if (!dead && !mbar_wait_bounded(&wbars[k % 3], (k / 3) & 1, kWaitLimitNs)) dead = true;
+    if (!dead && !mbar_wait_bounded(&wbars[k % NW], (k / NW) & 1, kWaitLimitNs)) dead = true;
+  };
+  auto slot_wait = [&](int k) {
+    if (!dead && !mbar_wait_bounded(&bars[k % NS], (k / NS) & 1, kWaitLimitNs)) dead = true;
   };
 
   if (!is_main) {
     // ------------------------------------------------------------ halo warps
+    // face crossed (0 W, 1 E, 2 S, 3 N); kind 0 nothing, 1 a neighbouring
+    // node whose populations enter, 2 a node at the wall whose own come back
     const int hid = tid - NTM;
-    int sx = 0, sy = 0, cell = 0, face = -1;  // source node, window cell, face crossed
+    using i0 = std::integral_constant<int, 0>;
+    using i1 = std::integral_constant<int, 1>;
+    using im = std::integral_constant<int, -1>;
+
+    // T: the type of this thread's values (rows: V, columns: R); face, kind,
+    // the column xl and window row r of the ring cell (kind 2: the node's own
+    // column, and r the row beyond the wall for rows); the node (kind 2); its
+    // coefficients in plane 0 (rows: in the fields, columns: an edge record)
+    auto run = [&](auto tag, auto col_tag, const int face, const int kind, const int xl, const int r, const int sx,
+                   const int sy, const R* const p0) {
+      using T = typename decltype(tag)::type;
+      constexpr bool COL = decltype(col_tag)::value;
+      constexpr bool ROW = !COL && NPT == 2;  // two nodes
+      // plane zb + p is copied to stage p % HD of this thread's own shared
+      // memory, HD - 2 planes ahead (a plane's time is about a loaded memory
+      // latency: with loads one plane ahead the whole CTA waited for them)
+      constexpr int HD = Sh::HD, HT = COL ? 2 * Sh::HCOL : HROW;
+      using R2 = typename std::conditional<sizeof(R) == 4, float2, double2>::type;
+      unsigned char* const stage0 = smem + Sh::OFF_HALO + (COL ? size_t(HD) * NC * HROW * sizeof(V) : 0);
+      const int ht = COL ? hid - HROW : hid;
+      auto fetch = [&](int p) {
+        const int z = zb + p;
+        if (kind != 0 && z <= ze) {
+          if constexpr (COL) {
+            const R2* g = reinterpret_cast<const R2*>(p0 + int64_t(ny) * NC * zwrap(z));
+            R2* h = reinterpret_cast<R2*>(stage0) + (p % HD) * (NC / 2) * HT + ht;
+#pragma unroll
+            for (int i = 0; i < NC / 2; ++i) cp_async<sizeof(R2)>(h + i * HT, g + i);
+          } else {
+            const char* g = reinterpret_cast<const char*>(p0 + plane * zwrap(z));
+            const uint32_t v32 = args.vol32;
+            T* h = reinterpret_cast<T*>(stage0) + (p % HD) * NC * HT + ht;
+#pragma unroll
+            for (int i = 0; i < NC; ++i)
+              cp_async<sizeof(T)>(h + i * HT, g + uint64_t(v32) * uint32_t(i * 32 * sizeof(R)));
+          }
+        }
+        cp_async_commit();
+      };
+      auto coef_of = [&](int p) {
+        T h[NC];
+        if constexpr (COL) {
+          const R2* hs = reinterpret_cast<const R2*>(stage0) + (p % HD) * (NC / 2) * HT + ht;
+#pragma unroll
+          for (int i = 0; i < NC; i += 2) {
+            const R2 v = hs[i / 2 * HT];
+            h[i] = v.x;
+            h[i + 1] = v.y;
+          }
+        } else {
+          const T* hs = reinterpret_cast<const T*>(stage0) + (p % HD) * NC * HT + ht;
+#pragma unroll
+          for (int i = 0; i < NC; ++i) h[i] = hs[i * HT];
+        }
+        Coef<T> k;
+        each_coef<L, T>(k, [&](auto I, T& v) { v = h[decltype(I)::value]; });
+        return k;
+      };
+      // bounce-back values of the node's descending links, for the next window
+      T held[Q];
+#pragma unroll
+      for (int a = 0; a < Q; ++a) held[a] = T(R(0));
+      // x sides a lane touches: bit 0 low, bit 1 high
+      auto x_walls = [&](int l) {
+        const int x = sx + l;
+        return args.per[0] ? 0 : (x == 0 ? 1 : 0) | (x == nx - 1 ? 2 : 0);
+      };
+      const int y_walls = args.per[1] ? 0 : (sy == 0 ? 1 : 0) | (sy == ny - 1 ? 2 : 0);
+      const int xw0 = x_walls(0), xw1 = ROW ? x_walls(1) : 0;
+
+      auto produce = [&](int p, auto AX, auto SG) {
+        constexpr int ax = decltype(AX)::value, sg = decltype(SG)::value;
+        R* win = win0 + (p % NW) * WSTRIDE;
+        if (kind == 1) {
+          const Coef<T> k = coef_of(p);
+          static_for<0, Q>([&](auto A_) {
+            constexpr int a = decltype(A_)::value;
+            if constexpr (comp<L>(ax, a) == sg) {
+              T v = post_v<L, a>(k);
+              R* w = win + Sh::off(a) + r * Sh::row(a);
+              if constexpr (L::cx(a) == 0) {
+                *reinterpret_cast<T*>(w + xl) = v;
+              } else if constexpr (ROW) {
+                w[xl / 2] = lane_of(v, 0);
+                if (xl + 1 < bxa) w[HB + 1 + xl / 2 + 1] = lane_of(v, 1);
+              } else {
+                w[Sh::col(xl)] = v;
+              }
+            }
+          });
+        } else if (kind == 2) {
+          const Coef<T> k = coef_of(p), kn = coef_of(p + 1);
+          static_for<0, Q>([&](auto A_) {
+            constexpr int a = decltype(A_)::value;
+            constexpr int cx = L::cx(a), cy = L::cy(a), cz = L::cz(a);
+            if constexpr (comp<L>(ax, a) == sg) {
+              // the link of this node through the wall: the node's own opposite
+              // population of the destination plane, c + cz
+              auto bounce = [&](const Coef<T>& kk) {
+                T v = post_v<L, L::opp(a)>(kk);
+                auto add = [&](int l, int xw) {
+                  int cb = 0;
+                  if constexpr (cx == 1) cb |= xw & 1;
+                  if constexpr (cx == -1) cb |= xw >> 1;
+                  if constexpr (cy == 1) cb |= (y_walls & 1) << 1;
+                  if constexpr (cy == -1) cb |= y_walls & 2;
+                  lane_of(v, l) = lane_of(v, l) + args.bb[a][cb];
+                };
+                add(0, xw0);
+                if constexpr (ROW) add(1, xw1);
+                return v;
+              };
+              T v;
+              if constexpr (cz == 0) v = bounce(k);
+              else if constexpr (cz == 1) v = bounce(kn);
+              else v = held[a];
+              if constexpr (cz == -1) held[a] = bounce(k);
+              R* w = win + Sh::off(a) + (ax == 1 ? r : r - cy) * Sh::row(a);
+              if constexpr (cx == 0) {
+                *reinterpret_cast<T*>(w + xl) = v;
+              } else if constexpr (ROW) {
+                // cells xl - cx and xl + 1 - cx
+                w[cx == 1 ? HB + 1 + xl / 2 : HB + 2 + xl / 2] = lane_of(v, 0);
+                if (xl + 1 < bxa) w[cx == 1 ? xl / 2 : xl / 2 + 1] = lane_of(v, 1);
+              } else {
+                w[Sh::col(xl - cx)] = v;
+              }
+            }
+          });
+        }
+      };
+      for (int p = 0; p < HD - 1; ++p) fetch(p);
+      for (int p = 0; p <= ze - zb; ++p) {
+        // into the stage plane p - 1 was read from; planes up to p + 1 landed
+        fetch(p + HD - 1);
+        cp_async_wait<HD - 2>();
+        if (face == 0) produce(p, i0{}, i1{});
+        else if (face == 1) produce(p, i0{}, im{});
+        if constexpr (NYF > 0) {
+          if (face == 2) produce(p, i1{}, i1{});
+          else if (face == 3) produce(p, i1{}, im{});
+        }
+        window_ready(p);
+        // plane p + 1's buffer must be free (see window_ready above)
+        if (p + 3 - NW >= 0) window_wait(p + 3 - NW);
+      }
+    };
+
     if (hid < HROW) {
-      const int i = hid % BX;
-      face = hid < BX ? 2 : 3;
-      sx = x0 + i;
-      sy = face == 2 ? y0 - 1 : y0 + bya;
-      cell = (face == 2 ? 0 : bya + 1) * WX + 1 + i;
-      if (i >= bxa) face = -1;
-    } else if (hid < HROW + 2 * WY) {
+      const int face = hid < HB ? 2 : 3;
+      const int xl = (hid % HB) * NPT;
+      const bool wall = face == 2 ? wallS : wallN;
+      int sy = face == 2 ? y0 - 1 : y0 + bya;
+      if (wall) sy = face == 2 ? y0 : y0 + bya - 1;  // the wall's own row
+      else sy = sy < 0 ? sy + ny : (sy >= ny ? sy - ny : sy);
+      run(type_tag<V>{}, std::false_type{}, face, xl < bxa ? (wall ? 2 : 1) : 0, xl, face == 2 ? 0 : bya + 1, x0 + xl,
+          sy, args.src + (x0 + xl) + args.pitch * sy);
+    } else {
       const int k = hid - HROW;
-      const int r = k % WY;
-      face = k < WY ? 0 : 1;
-      sx = face == 0 ? x0 - 1 : x0 + bxa;
-      sy = y0 - PY + r;
-      cell = r * WX + (face == 0 ? 0 : bxa + 1);
-      if (r >= bya + 2 * PY) face = -1;
-    }
-    // periodic images; beyond a wall nothing is ever pulled from
-    if (sx < 0 || sx >= nx) {
-      if (args.per[0]) sx = sx < 0 ? sx + nx : sx - nx;
-      else face = -1;
-    }
-    if (sy < 0 || sy >= ny) {
-      if (args.per[1]) sy = sy < 0 ? sy + ny : sy - ny;
-      else face = -1;
-    }
-    const R* p0 = args.src + sx + args.pitch * sy;
-    R h[NC];
-#pragma unroll
-    for (int i = 0; i < NC; ++i) h[i] = R(0);
-    auto fetch = [&](int z) {
-      if (face >= 0 && z <= ze) {
-        const R* p = p0 + plane * zwrap(z);
-#pragma unroll
-        for (int i = 0; i < NC; ++i) {
-          h[i] = *p;
-          p += args.vol;
+      const int r = k % Sh::HCOL, yl = r - PY;
+      const int face = k < Sh::HCOL ? 0 : 1;
+      const bool wall = face == 0 ? wallW : wallE;
+      // the neighbouring tile's last or first column, or at a wall this tile's
+      // own first or last
+      const int side = wall ? face : 1 - face;
+      const int tc = wall ? tI : (face == 0 ? (tI > 0 ? tI : args.ntx) - 1 : (tI + 1 < args.ntx ? tI + 1 : 0));
+      int sy = y0 + yl;
+      int kind = r < WY ? (wall ? 2 : 1) : 0;
+      if (wall) {
+        if (yl < 0 || yl >= bya) kind = 0;
+      } else {
+        if (yl > bya - 1 + PY) kind = 0;
+        // a corner beyond a y wall belongs to that wall's nodes
+        if (sy < 0 || sy >= ny) {
+          if (args.per[1]) sy = sy < 0 ? sy + ny : sy - ny;
+          else kind = 0;
         }
       }
-    };
-    auto produce = [&](int c) {
-      R* win = win0 + ((c - zb) % 3) * WSTRIDE + cell;
-      Coef<R> k;
-      each_coef<L, R>(k, [&](auto I, R& v) { v = h[decltype(I)::value]; });
-      fetch(c + 1);
-      auto put = [&](auto AX, auto SG) {
-        constexpr int ax = decltype(AX)::value, sg = decltype(SG)::value;
-        static_for<0, Q>([&](auto A_) {
-          constexpr int a = decltype(A_)::value;
-          if constexpr (comp<L>(ax, a) == sg) win[lat_index<L>(a) * WPLANE] = post<L, R, a>(k);
-        });
-      };
-      using i0 = std::integral_constant<int, 0>;
-      using i1 = std::integral_constant<int, 1>;
-      using im = std::integral_constant<int, -1>;
-      if (face == 0) put(i0{}, i1{});
-      else if (face == 1) put(i0{}, im{});
-      if constexpr (NYF > 0) {
-        if (face == 2) put(i1{}, i1{});
-        else if (face == 3) put(i1{}, im{});
-      }
-    };
-    fetch(zb);
-    for (int c = zb; c <= ze; ++c) {
-      produce(c);
-      window_ready(c - zb);
-      window_wait(c - zb);
+      if (kind == 0) sy = 0;
+      // the ring column, or at a wall the column of the node itself
+      const int xl = face == 0 ? (wall ? 0 : -1) : (wall ? bxa - 1 : bxa);
+      run(type_tag<R>{}, std::true_type{}, face, kind, xl, r, x0 + xl, sy,
+          args.esrc + k3_edge(side, tc, args.ntx, int64_t(ny) * nz, sy) * NC);
     }
     if (dead) atomicExch(args.status, LB_E_TIMEOUT);
     return;
   }
 
   // -------------------------------------------------------------- node warps
-  const int tx = tid % BX, ty = tid / BX;
-  const int x = x0 + tx, y = y0 + ty;
-  const bool active = tx < bxa && ty < bya;
-  const bool bxlo = x == 0 && !args.per[0];
-  const bool bxhi = x == nx - 1 && !args.per[0];
-  const bool bylo = y == 0 && !args.per[1];
-  const bool byhi = y == ny - 1 && !args.per[1];
-  const bool xy_wall = bxlo || bxhi || bylo || byhi;
+  const int i = tid % HB, ty = tid / HB;
+  const int x = x0 + NPT * i, y = y0 + ty;
+  const bool active = NPT * i < bxa && ty < bya;
+  const bool act1 = NPT * i + 1 < bxa;  // the pair's second node
   const bool z_walls = !args.per[2];
-  const int wbase = (ty + PY) * WX + (tx + 1);
+  // this thread's place in the rows of the two kinds of directions
+  const int b0 = (ty + PY) * BX + NPT * i;
+  const int bm = (ty + PY) * RM + i;
   R* const out0 = args.dst + x + args.pitch * y;
-
+  // edge records this thread writes: of the tile's first column (its node 0)
+  // and last column (node eastl)
+  const bool west = i == 0, east = NPT * i < bxa && NPT * (i + 1) >= bxa;
+  const int eastl = bxa - 1 - NPT * i;
+  R* const edge0 = args.edst + k3_edge(west ? 0 : 1, tI, args.ntx, int64_t(ny) * nz, y) * NC;
   constexpr int zm = nonlateral_dir<L, -1>(), zp = nonlateral_dir<L, 1>();
+
+  auto put = [&](R* win, auto A_, V v) {
+    constexpr int a = decltype(A_)::value;
+    if constexpr (L::cx(a) == 0) {
+      *reinterpret_cast<V*>(win + Sh::off(a) + b0) = v;
+    } else if constexpr (NPT == 2) {
+      win[Sh::off(a) + bm] = lane_of(v, 0);
+      if (act1) win[Sh::off(a) + bm + HB + 2] = lane_of(v, 1);
+    } else {
+      win[Sh::off(a) + bm + 1] = lane_of(v, 0);
+    }
+  };
+  // the values of direction a at the thread's nodes shifted by (-dx, -dy)
+  auto get = [&](const R* win, auto A_, auto DX, auto DY) -> V {
+    constexpr int a = decltype(A_)::value, dx = decltype(DX)::value, dy = decltype(DY)::value;
+    if constexpr (L::cx(a) == 0) {
+      return *reinterpret_cast<const V*>(win + Sh::off(a) + b0 - dy * BX);
+    } else {
+      const R* w = win + Sh::off(a) + bm - dy * RM;
+      V v;
+      if constexpr (NPT == 2) {
+        lane_of(v, 0) = w[dx == 0 ? 0 : (dx == 1 ? HB + 1 : HB + 2)];
+        lane_of(v, 1) = w[dx == 0 ? HB + 2 : (dx == 1 ? 0 : 1)];
+      } else {
+        v = w[1 - dx];
+      }
+      return v;
+    }
+  };
+
   // collide plane c = zb + k: the laterally moving populations go to the window, the
   // others to their destinations (rest: plane c, -z: c - 1, +z: c + 1)
-  auto produce = [&](int k, R& rest, R& down, R& up) {
-    const int slot = k % NS;
-    if (!dead && !mbar_wait_bounded(&bars[slot], (k / NS) & 1, kWaitLimitNs)) dead = true;
+  auto produce = [&](int k, R* win, V& rest, V& down, V& up) {
+    slot_wait(k);
     if (active) {
-      R* win = win0 + (k % 3) * WSTRIDE + wbase;
-      const R* sl = slots + size_t(slot) * NC * NTM + tid;
-      Coef<R> kc;
-      each_coef<L, R>(kc, [&](auto I, R& v) { v = sl[decltype(I)::value * NTM]; });
-      rest = post<L, R, 0>(kc);
-      static_for<0, n_pairs<L>()>([&](auto P) {
-        constexpr int a = pair_first<L>(decltype(P)::value);
+      const R* sl = slots + (k % NS) * SLOTN + NPT * tid;
+      Coef<V> kc;
+      each_coef<L, V>(kc, [&](auto I, V& v) { v = *reinterpret_cast<const V*>(sl + decltype(I)::value * (BX * BY)); });
+      rest = post_v<L, 0>(kc);
+      static_for<1, Q>([&](auto A_) {
+        constexpr int a = decltype(A_)::value;
         constexpr int b = L::opp(a);
-        constexpr R w = R(weight<L>(a));
-        R even, wodd;
-        post_parts<L, R, a>(kc, even, wodd);
-        const R fa = fma_r(w, even, wodd), fb = fma_r(w, even, -wodd);
-        if constexpr (is_lateral<L>(a)) {
-          win[lat_index<L>(a) * WPLANE] = fa;
-          win[lat_index<L>(b) * WPLANE] = fb;
-        } else {
-          (a == zp ? up : down) = fa;
-          (b == zp ? up : down) = fb;
+        if constexpr (leading_sign<L>(a) == 1) {
+          V fa, fb;
+          post_pair<L, a>(kc, fa, fb);
+          if constexpr (is_lateral<L>(a)) {
+            put(win, A_, fa);
+            put(win, std::integral_constant<int, b>{}, fb);
+          } else {
+            static_assert(a == zp && b == zm, "the pair along z");
+            up = fa;
+            down = fb;
+          }
         }
       });
     }
   };
 
-  // load plane zb + k + NS into the slot of plane zb + k (thread 0)
-  auto refill = [&](int k) {
-    uint64_t* bar = &bars[k % NS];
-    mbar_arrive_expect_tx(bar, static_cast<uint32_t>(Sh::SLOT));
-    tma_load_4d(slots + size_t(k % NS) * NC * NTM, tmap_p, x0, y0, zwrap(zb + k + NS), 0, bar);
-    ++issued;
-  };
-
   // gathered populations of three destination planes; the roles of the sets
   // are permuted at compile time
-  R G[3][Q];
-  produce(0, G[1][0], G[0][zm], G[2][zp]);
+  V G[3][Q];
+  produce(0, win0, G[1][0], G[0][zm], G[2][zp]);
   window_ready(0);
   window_wait(0);
 
@@ -290,17 +513,16 @@ __device__ __forceinline__ void k3_brick(const CUtensorMap* tmap_p, const K3Args
     constexpr int k = decltype(K)::value;
     const int g = zb + 3 * t + k;
     const int kc = 3 * t + k + 1;  // plane c's index
-    R(&G0)[Q] = G[k % 3];        // destination plane g - 1
-    R(&G1)[Q] = G[(k + 1) % 3];  // g
-    R(&G2)[Q] = G[(k + 2) % 3];  // g + 1
+    V(&G0)[Q] = G[k % 3];          // destination plane g - 1
+    V(&G1)[Q] = G[(k + 1) % 3];    // g
+    V(&G2)[Q] = G[(k + 2) % 3];    // g + 1
     const int c = g + 1;
-    const R* win_g = win0 + k * WSTRIDE + wbase;
-    R* win_c = win0 + ((k + 1) % 3) * WSTRIDE + wbase;
-    R up_c = R(0);  // plane c's +z population: of plane c + 1, whose set is G0
-    const R down_g = G0[zm], up_g = G2[zp];  // this node's own, for a z wall's bounce-back
-    const bool z_lo = z_walls && g == 0, z_hi = z_walls && g == nz - 1;
+    const R* win_g = win0 + (kc - 1) % NW * WSTRIDE;
+    R* win_c = win0 + kc % NW * WSTRIDE;
+    V up_c = V(R(0));  // plane c's +z population: of plane c + 1, whose set is G0
+    const V down_g = G0[zm], up_g = G2[zp];  // this node's own, for a z wall's bounce-back
     if (c <= ze) {
-      produce(kc, G2[0], G1[zm], up_c);
+      produce(kc, win_c, G2[0], G1[zm], up_c);
       window_ready(kc);
     }
 
@@ -310,38 +532,37 @@ __device__ __forceinline__ void k3_brick(const CUtensorMap* tmap_p, const K3Args
           constexpr int a = decltype(A_)::value;
           constexpr int cx = L::cx(a), cy = L::cy(a), cz = L::cz(a);
           if constexpr (is_lateral<L>(a)) {
-            const R v = win_g[lat_index<L>(a) * WPLANE - cy * WX - cx];
+            const V v = get(win_g, A_, std::integral_constant<int, cx>{}, std::integral_constant<int, cy>{});
             if constexpr (cz == -1) G0[a] = v;
             if constexpr (cz == 0) G1[a] = v;
             if constexpr (cz == 1) G2[a] = v;
           }
         });
-        // halfway bounce-back for destination plane g (threads next to a wall)
-        if (xy_wall || z_lo || z_hi) {
+        // halfway bounce-back at a z wall
+        if (z_walls && (g == 0 || g == nz - 1)) {
+          const bool z_lo = g == 0, z_hi = g == nz - 1;
           static_for<1, Q>([&](auto A_) {
             constexpr int a = decltype(A_)::value;
             constexpr int cx = L::cx(a), cy = L::cy(a), cz = L::cz(a);
-            int cb = 0;
-            if constexpr (cx == 1) cb |= bxlo ? 1 : 0;
-            if constexpr (cx == -1) cb |= bxhi ? 1 : 0;
-            if constexpr (cy == 1) cb |= bylo ? 2 : 0;
-            if constexpr (cy == -1) cb |= byhi ? 2 : 0;
-            if constexpr (cz == 1) cb |= z_lo ? 4 : 0;
-            if constexpr (cz == -1) cb |= z_hi ? 4 : 0;
-            if (cb != 0) {
-              constexpr int oa = L::opp(a);
-              R back;
-              if constexpr (is_lateral<L>(oa)) back = win_g[lat_index<L>(oa) * WPLANE];
-              else back = oa == zm ? down_g : up_g;
-              const R v = back + args.bb[a][cb];
-              // a descending link is gathered with plane c: its value waits in
-              // the window cell it would be pulled from, which lies beyond the
-              // wall and has no other writer or reader (beyond a z wall no
-              // plane c is gathered)
-              if constexpr (cz == -1 && is_lateral<L>(a)) {
-                if (z_hi) G1[a] = v;
-                else win_c[lat_index<L>(a) * WPLANE - cy * WX - cx] = v;
-              } else {
+            if constexpr (cz != 0) {
+              if (cz == 1 ? z_lo : z_hi) {
+                constexpr int oa = L::opp(a);
+                V v;
+                if constexpr (is_lateral<L>(oa))
+                  v = get(win_g, std::integral_constant<int, oa>{}, std::integral_constant<int, 0>{},
+                          std::integral_constant<int, 0>{});
+                else
+                  v = oa == zm ? down_g : up_g;
+                int cb = 4;
+                if constexpr (cy == 1) cb |= y == 0 && !args.per[1] ? 2 : 0;
+                if constexpr (cy == -1) cb |= y == ny - 1 && !args.per[1] ? 2 : 0;
+#pragma unroll
+                for (int l = 0; l < NPT; ++l) {
+                  int cl = cb;
+                  if constexpr (cx == 1) cl |= x + l == 0 && !args.per[0] ? 1 : 0;
+                  if constexpr (cx == -1) cl |= x + l == nx - 1 && !args.per[0] ? 1 : 0;
+                  lane_of(v, l) = lane_of(v, l) + args.bb[a][cl];
+                }
                 G1[a] = v;
               }
             }
@@ -351,31 +572,41 @@ __device__ __forceinline__ void k3_brick(const CUtensorMap* tmap_p, const K3Args
       // plane g - 1 is complete: collide it
       const int zd = g - 1;
       if (zd >= z0) {
-        R fr[Q];
+        V fr[Q];
         static_for<0, Q>([&](auto A_) {
           constexpr int a = decltype(A_)::value;
-          fr[a] = round_to_storage<S, R>(G0[a]);
+          fr[a] = round_value<S>(G0[a]);
         });
-        Mom<R> m;
-        moments<L, R, FORCE>(fr, args.ph, m);
-        Coef<R> kc;
-        coeffs<L, R, FORCE>(m, args.ph, kc);
+        Coef<V> kc2;
+        moments_coeffs<L, FORCE>(fr, args.ph, kc2);
         char* o = reinterpret_cast<char*>(out0 + plane * zd);
         const uint32_t v32 = args.vol32;
-        each_coef<L, R>(kc, [&](auto I, R& v) {
-          *reinterpret_cast<R*>(o + uint64_t(v32) * uint32_t(decltype(I)::value * 32 * sizeof(R))) = v;
-        });
+        if (NPT == 1 || act1) {
+          each_coef<L, V>(kc2, [&](auto I, V& v) {
+            *reinterpret_cast<V*>(o + uint64_t(v32) * uint32_t(decltype(I)::value * 32 * sizeof(R))) = v;
+          });
+        } else {
+          each_coef<L, V>(kc2, [&](auto I, V& v) {
+            *reinterpret_cast<R*>(o + uint64_t(v32) * uint32_t(decltype(I)::value * 32 * sizeof(R))) = lane_of(v, 0);
+          });
+        }
+        if (west || east) {
+          R* e = edge0 + int64_t(ny) * NC * zd;
+          put_record<L>(kc2, e, west ? 0 : eastl);
+          // a tile of one column pair is both
+          if (west && east) put_record<L>(kc2, e + int64_t(args.ntx) * ny * nz * NC, eastl);
+        }
       }
     }
     G0[zp] = up_c;
     if (c <= ze) {
       window_wait(kc);
       // every thread has read plane c's slot
-      if (tid == 0 && !dead && c + NS <= ze) refill(kc);
+      if (tid == 0 && !dead && c + NS <= ze) load_plane(kc + NS);
     }
   };
   // the slot of plane zb is free once its window is complete
-  if (tid == 0 && !dead && zb + NS <= ze) refill(0);
+  if (tid == 0 && !dead && zb + NS <= ze) load_plane(NS);
   // gathers planes zb .. ze, completes planes z0 .. z1 - 1 (the last trip,
   // g = z1, only completes where plane z1 does not exist)
   const int trips = z1 - zb + 1;
@@ -399,33 +630,38 @@ __device__ __forceinline__ void k3_brick(const CUtensorMap* tmap_p, const K3Args
   }
 }
 
-template <class L, class S, class R, int BX, int BY, int NS, bool FORCE, int MINB>
-__global__ void __launch_bounds__(K3Shape<L, R, BX, BY, NS, MINB>::NT, MINB)
-    k3_step(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ K3Args<R> args) {
+template <class L, class S, class R, int BX, int BY, int NS, int NPT, bool FORCE, int MINB>
+__global__ void __launch_bounds__(K3Shape<L, R, BX, BY, NS, NPT, MINB>::NT, MINB)
+    k3_step(const __grid_constant__ CUtensorMap tmap,
+            const __grid_constant__ K3Args<R, typename K3Shape<L, R, BX, BY, NS, NPT, MINB>::V> args) {
   const int b = blockIdx.x;
-  k3_brick<L, S, R, BX, BY, NS, FORCE, MINB>(&tmap, args, b % args.ntx, (b / args.ntx) % args.nty,
-                                             b / (args.ntx * args.nty));
+  k3_brick<L, S, R, BX, BY, NS, NPT, FORCE, MINB>(&tmap, args, b % args.ntx, (b / args.ntx) % args.nty,
+                                                  b / (args.ntx * args.nty));
 }
 
-// Populations -> coefficient fields, node by node (each thread reads all of
-// its node's populations before it writes, so the fields may lie in the
-// population array).
+// Populations -> coefficient fields and edge records, node by node (each thread
+// reads all of its node's populations before it writes, so the fields may lie
+// in the population array).  bx: the tile width the edge records are for.
 template <class L, class S, class R, bool FORCE>
-__global__ void __launch_bounds__(256) k3_enter(const S* f, R* dst, int64_t vol, int nx, int pitch, Phys<R> ph) {
+__global__ void __launch_bounds__(256)
+    k3_enter(const S* f, R* dst, R* edst, int64_t vol, int nx, int64_t rows, int pitch, int bx, Phys<R> ph) {
   for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < vol; i += int64_t(gridDim.x) * blockDim.x) {
     // rows are whole 32-element segments; the padding of a row stays zero
-    const uint32_t seg = uint32_t(i >> 5) % uint32_t(pitch >> 5);
-    if (int(seg * 32 + (i & 31)) >= nx) continue;
+    const uint32_t segs = uint32_t(pitch >> 5), seg = uint32_t(i >> 5), row = seg / segs;
+    const int x = int((seg - row * segs) * 32 + uint32_t(i & 31));
+    if (x >= nx) continue;
     R fr[L::Q];
     static_for<0, L::Q>([&](auto A_) {
       constexpr int a = decltype(A_)::value;
       fr[a] = load_as<S, R>(f[a * vol + i]);
     });
-    Mom<R> m;
-    moments<L, R, FORCE>(fr, ph, m);
     Coef<R> kc;
-    coeffs<L, R, FORCE>(m, ph, kc);
+    moments_coeffs<L, FORCE>(fr, ph, kc);
     each_coef<L, R>(kc, [&](auto I, R& v) { dst[decltype(I)::value * vol + i] = v; });
+    const int tI = x / bx, xl = x - tI * bx, ntx = (nx + bx - 1) / bx;
+    constexpr int NC = n_coef<L>();
+    if (xl == 0) put_record<L>(kc, edst + k3_edge(0, tI, ntx, rows, row) * NC, 0);
+    if (xl == bx - 1 || x == nx - 1) put_record<L>(kc, edst + k3_edge(1, tI, ntx, rows, row) * NC, 0);
   }
 }
 

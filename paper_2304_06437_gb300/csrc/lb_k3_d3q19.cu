@@ -1,13 +1,14 @@
 // lb_k3_d3q19.cu -- compiled tiles of the step in moment form for D3Q19.
-// Each entry: storage / arithmetic type, tile bx x by, TMA ring depth, CTAs
-// per SM; and the brick cross-sections whose contexts can end a run.
+// Each entry: storage / arithmetic type, tile bx x by, TMA ring depth, nodes
+// per thread, CTAs per SM; and the brick cross-sections whose contexts can end a run.
 #include "lb_k3_launch.cuh"
 
 namespace lbgb {
 
 extern const K3Variant k3_variants_d3q19[] = {
-    K3Impl<D3Q19, float, float, 32, 16, 3, 1>::variant(LB_D3Q19, LB_F32),
-    K3Impl<D3Q19, double, double, 32, 8, 2, 1>::variant(LB_D3Q19, LB_F64),
+    K3Impl<D3Q19, float, float, 32, 16, 3, 1, 1>::variant(LB_D3Q19, LB_F32),
+    K3Impl<D3Q19, float, float, 32, 4, 2, 1, 2>::variant(LB_D3Q19, LB_F32),  // small domains
+    K3Impl<D3Q19, double, double, 32, 8, 2, 1, 1>::variant(LB_D3Q19, LB_F64),
 };
 extern const int k3_n_variants_d3q19 = sizeof(k3_variants_d3q19) / sizeof(k3_variants_d3q19[0]);
 

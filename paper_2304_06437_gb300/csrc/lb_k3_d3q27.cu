@@ -1,13 +1,13 @@
 // lb_k3_d3q27.cu -- compiled tiles of the step in moment form for D3Q27.
-// Each entry: storage / arithmetic type, tile bx x by, TMA ring depth, CTAs
-// per SM; and the brick cross-sections whose contexts can end a run.
+// Each entry: storage / arithmetic type, tile bx x by, TMA ring depth, nodes
+// per thread, CTAs per SM; and the brick cross-sections whose contexts can end a run.
 #include "lb_k3_launch.cuh"
 
 namespace lbgb {
 
 extern const K3Variant k3_variants_d3q27[] = {
-    K3Impl<D3Q27, float, float, 32, 12, 3, 1>::variant(LB_D3Q27, LB_F32),
-    K3Impl<D3Q27, double, double, 32, 6, 2, 1>::variant(LB_D3Q27, LB_F64),
+    K3Impl<D3Q27, float, float, 32, 12, 3, 1, 1>::variant(LB_D3Q27, LB_F32),
+    K3Impl<D3Q27, double, double, 32, 6, 2, 1, 1>::variant(LB_D3Q27, LB_F64),
 };
 extern const int k3_n_variants_d3q27 = sizeof(k3_variants_d3q27) / sizeof(k3_variants_d3q27[0]);
 

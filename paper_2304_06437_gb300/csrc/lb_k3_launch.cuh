@@ -2,6 +2,8 @@
 // per compiled tile shape, and of the brick launches that end a run.
 #pragma once
 
+#include <algorithm>
+
 #include "lb_k1_launch.cuh"
 #include "lb_k3.cuh"
 
@@ -9,7 +11,7 @@ namespace lbgb {
 
 // A compiled tile of k3_step (lattice x storage x bx x by).
 struct K3Variant {
-  int lattice, storage, bx, by, ns, minb;
+  int lattice, storage, bx, by, ns, npt, minb;
   cudaError_t (*configure)();
   // one step of the context's domain: set src (0 = A, 1 = B) to the other
   cudaError_t (*step)(lb_ctx*, int src);
@@ -29,15 +31,16 @@ struct LeaveVariant {
 template <class L>
 LB_HD constexpr int coef_set_b() { return L::D == 2 ? 6 : 10; }
 
-template <class L, class S, class R, int BX, int BY, int NS, int MINB>
+template <class L, class S, class R, int BX, int BY, int NS, int NPT, int MINB>
 struct K3Impl {
-  using Sh = K3Shape<L, R, BX, BY, NS, MINB>;
+  using Sh = K3Shape<L, R, BX, BY, NS, NPT, MINB>;
+  using V = typename Sh::V;
 
   static cudaError_t configure() {
-    cudaError_t e = cudaFuncSetAttribute(k3_step<L, S, R, BX, BY, NS, false, MINB>,
+    cudaError_t e = cudaFuncSetAttribute(k3_step<L, S, R, BX, BY, NS, NPT, false, MINB>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, int(Sh::SMEM));
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k3_step<L, S, R, BX, BY, NS, true, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      e = cudaFuncSetAttribute(k3_step<L, S, R, BX, BY, NS, NPT, true, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                int(Sh::SMEM));
     return e;
   }
@@ -46,10 +49,15 @@ struct K3Impl {
     return static_cast<R*>(ctx->f) + (which ? int64_t(coef_set_b<L>()) * ctx->g.vol : 0);
   }
 
+  // the edge records of a set, after the two sets (moment_scratch_elems)
+  static R* edges(lb_ctx* ctx, int which) {
+    return static_cast<R*>(ctx->f) + moment_edge_at(ctx->g) + which * moment_edge_elems(ctx->g, BX);
+  }
+
   static cudaError_t step(lb_ctx* ctx, int src) {
     const Geometry& g = ctx->g;
-    K3Args<R> a;
-    a.ph = make_phys<R>(g);
+    K3Args<R, V> a;
+    a.ph = make_phys<V>(g);
     a.nx = g.nx;
     a.ny = g.ny;
     a.nz = g.nz;
@@ -63,16 +71,18 @@ struct K3Impl {
     a.ntz = div_up(g.nz, a.bz);
     a.src = coef_set(ctx, src);
     a.dst = coef_set(ctx, 1 - src);
+    a.esrc = edges(ctx, src);
+    a.edst = edges(ctx, 1 - src);
     a.status = ctx->d_status;
     for (int i = 0; i < 27; ++i)
       for (int j = 0; j < 8; ++j) a.bb[i][j] = R(0);
     make_bounce_terms<L, R>(g, a.bb);
     const int grid = a.ntx * a.nty * a.ntz;
-    const CUtensorMap& tm = src ? ctx->mr.tmap_b : ctx->mr.tmap_a;
+    const CUtensorMap& tm = ctx->mr.maps[src];
     if (g.has_force)
-      k3_step<L, S, R, BX, BY, NS, true, MINB><<<grid, Sh::NT, Sh::SMEM, ctx->stream>>>(tm, a);
+      k3_step<L, S, R, BX, BY, NS, NPT, true, MINB><<<grid, Sh::NT, Sh::SMEM, ctx->stream>>>(tm, a);
     else
-      k3_step<L, S, R, BX, BY, NS, false, MINB><<<grid, Sh::NT, Sh::SMEM, ctx->stream>>>(tm, a);
+      k3_step<L, S, R, BX, BY, NS, NPT, false, MINB><<<grid, Sh::NT, Sh::SMEM, ctx->stream>>>(tm, a);
     return cudaGetLastError();
   }
 
@@ -80,17 +90,18 @@ struct K3Impl {
     const Geometry& g = ctx->g;
     const int64_t blocks = std::min<int64_t>((g.vol + 255) / 256, int64_t(1) << 30);
     const S* f = static_cast<const S*>(ctx->f);
+    const int64_t rows = int64_t(g.ny) * g.nz;
     if (g.has_force)
-      k3_enter<L, S, R, true><<<int(blocks), 256, 0, ctx->stream>>>(f, coef_set(ctx, dst), g.vol, g.nx, int(g.pitch),
-                                                                    make_phys<R>(g));
+      k3_enter<L, S, R, true><<<int(blocks), 256, 0, ctx->stream>>>(f, coef_set(ctx, dst), edges(ctx, dst), g.vol, g.nx,
+                                                                    rows, int(g.pitch), BX, make_phys<R>(g));
     else
-      k3_enter<L, S, R, false><<<int(blocks), 256, 0, ctx->stream>>>(f, coef_set(ctx, dst), g.vol, g.nx, int(g.pitch),
-                                                                     make_phys<R>(g));
+      k3_enter<L, S, R, false><<<int(blocks), 256, 0, ctx->stream>>>(f, coef_set(ctx, dst), edges(ctx, dst), g.vol,
+                                                                     g.nx, rows, int(g.pitch), BX, make_phys<R>(g));
     return cudaGetLastError();
   }
 
   static constexpr K3Variant variant(int lattice, int storage) {
-    return K3Variant{lattice, storage, BX, BY, NS, MINB, &configure, &step, &enter};
+    return K3Variant{lattice, storage, BX, BY, NS, NPT, MINB, &configure, &step, &enter};
   }
 };
 

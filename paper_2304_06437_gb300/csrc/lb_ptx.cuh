@@ -78,6 +78,20 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
   }
 }
 
+// per-thread asynchronous copy of N bytes (4, 8 or 16) global -> shared; the
+// copies issued since the last commit form a group, and groups complete in
+// order
+template <int N>
+__device__ __forceinline__ void cp_async(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_addr(dst)), "l"(src), "n"(N) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// wait until at most N of this thread's groups are in flight
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
 // order this thread's generic-proxy shared-memory accesses before later
 // async-proxy (TMA) accesses to the same shared memory
 __device__ __forceinline__ void fence_proxy_async_smem() {
