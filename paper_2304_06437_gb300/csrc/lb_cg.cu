@@ -1,18 +1,17 @@
 // lb_cg.cu -- two-component colour-gradient step (paper section 2.1) in the
-// thread-safe form of section 4: moments are taken in one launch, the phase
-// field gradient in a second, and a third rebuilds each colour's populations
-// at every node by pulling the post-collision set of the upstream node from
-// those moment fields.  No launch reads and writes the same population, so
-// each colour keeps ONE population array.
+// thread-safe form of section 4: a node's post-collision set is known from a
+// few moment fields, the phase field gradient is taken in a launch of its own,
+// and a node's new populations are pulled from the fields of its upstream
+// nodes.
 //
-// Per node x (moments launch), from the two colours f_R, f_B:
+// Per node x, from the two colours f_R, f_B:
 //   rho_R = sum f_R, rho_B = sum f_B, g = f_R + f_B, and the regularized
 //   relaxation coefficients of g (lb_collide.cuh: A, B, C, the order-2
 //   Hermite form of Eq. LBexp / Eq. hermite), phi = (rho_R - rho_B) / rho,
 //   c_R = rho_R / rho and c_RB = beta rho_R rho_B / rho;
 // (gradient launch) grad phi = (1/cs2) sum_a t_a c_a phi(x + c_a), stored as
 //   |grad phi| and the unit normal n;
-// (rebuild launch) for every direction a and upstream node x = y - c_a:
+// (pull) for every direction a and upstream node x = y - c_a:
 //   g*_a = t_a (A + B.c_a + c_a.C.c_a) + (9/4) sigma omega |grad phi|
 //          [t_a (c_a.n)^2 - B_a]                          (perturbation)
 //   f_R(y)_a = c_R g*_a + c_RB t_a (c_a.n)/|c_a|,  f_B(y)_a = g*_a - f_R(y)_a
@@ -21,6 +20,29 @@
 // so that g is stored shifted by t_a rho0 as in the single-component path.
 // Periodic box only; D2Q9 and D3Q19; FP64 or FP32 storage and arithmetic.
 //
+// Between two steps of one lb_cg_step() call the populations exist in
+// registers only: the step launch pulls them from one set of fields and writes
+// the moment fields of the next set.  A run is
+//   enter (populations -> set A), gradient A,
+//   n - 1 times: step (A -> B or B -> A), gradient of the new set,
+//   leave (set A -> populations),
+// two launches a step.  Set A has memory of its own; set B lies in the
+// population arrays, which the enter launch has read by then, so a run needs an
+// odd n (an even one is preceded by a run of one step).  The arithmetic is that of
+// populations written and read back at every step, operation by operation.
+//
+// Layout of a set: quads, 16-byte groups (FP32) of four values of a node, so
+// that a pull is 3 (2D) or 4 (3D) vector loads a direction: the coefficients
+// with c_R and c_RB behind them, and |grad phi| with n; and phi on its own,
+// which the gradient reads at 8 or 18 neighbours.  FP32 bytes per update: the
+// step reads 48 and writes 36 (3D: 64 and 52), the gradient reads 4 and writes
+// 16: 104 (136), where three launches over populations and planar fields moved
+// 284 (444).  Measured per step on one GB300, three launches against this form:
+// D2Q9 FP32 4096^2 1126 -> 488 us, 2048 x 1536 with near-contact forces 328 ->
+// 137 us, D3Q19 FP32 192^3 933 -> 766 us (bound by the L1's loads of a pull),
+// 97 x 61 x 113 98.6 -> 76.5 us; FP64 is bound by its arithmetic (1024^2 624 ->
+// 613 us).
+//
 // Near-contact interactions (section 2.2), when switched on: the gradient
 // launch also flags node y if, for some direction a, the node y - h c_a is
 // bulk (phi < -1 + eps) and both y and y - 2h c_a are not -- the paper's test
@@ -28,8 +50,10 @@
 // writes only its own node -- and a flagged node's relaxation coefficients
 // are recomputed from its own populations with the body force
 // F = A rho_R grad phi / |grad phi| (the forcing of the single-component
-// step).  No thread reads coefficients in that launch, and populations are
-// only written by the rebuild launch after it.
+// step).  Its populations are those in memory at a run's first step, and are
+// pulled once more from the set before at the others (flagged nodes line the
+// thin films between droplets: few).  No thread reads this set's coefficients
+// in that launch, and the set before is only written by the launch after it.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -43,21 +67,53 @@ namespace lbgb {
 namespace {
 
 constexpr int kCgThreads = 256;
-// per-node fields of the moments launch: 10 relaxation coefficients, c_R,
-// c_RB, phi; of the gradient launch: |grad phi| and n (3)
-constexpr int kCgFields = 17;
-enum { F_COEF = 0, F_CR = 10, F_CRB = 11, F_PHI = 12, F_GN = 13, F_N = 14 };
+// values per node of a set: NC coefficients, c_R, c_RB; |grad phi| and n (3); phi
+constexpr int kCgFields = 17;  // of D3Q19; D2Q9 uses 13
 
-struct CgGeom {
-  int nx, ny, nz;  // internal axes (2D: nx x 1 x ny)
-  int64_t n;
+template <class R>
+struct alignas(16) Quad {
+  R v[4];
 };
 
-__device__ __forceinline__ int64_t cg_wrap_index(const CgGeom& g, int x, int y, int z) {
+// one set of fields; quad j of node i is k[j * n + i]
+template <class R>
+struct CgSet {
+  Quad<R>* k;     // the coefficients in the order of each_coef, c_R, c_RB
+  Quad<R>* grad;  // |grad phi|, n
+  R* phi;
+};
+
+// Extents, and the box of nodes a thread block works on: 2^lx x 2^ly x 2^lz =
+// kCgThreads nodes (internal axes; 2D: nx x 1 x ny).
+struct CgGeom {
+  int nx, ny, nz;
+  int64_t n;
+  int lx, ly, lz;
+  uint32_t ntx, nty, ntz;  // boxes along each axis
+};
+
+struct CgNode {
+  int x, y, z;
+  bool in;
+};
+__device__ __forceinline__ CgNode cg_node(const CgGeom& g) {
+  const uint32_t b = blockIdx.x, r = b / g.ntx;
+  CgNode o;
+  o.x = int((b - r * g.ntx) << g.lx) + int(threadIdx.x & ((1u << g.lx) - 1));
+  const uint32_t bz = r / g.nty;
+  o.y = int((r - bz * g.nty) << g.ly) + int((threadIdx.x >> g.lx) & ((1u << g.ly) - 1));
+  o.z = int(bz << g.lz) + int(threadIdx.x >> (g.lx + g.ly));
+  o.in = o.x < g.nx && o.y < g.ny && o.z < g.nz;
+  return o;
+}
+
+// node index, for coordinates up to one period outside (a domain that fits the
+// memory has fewer than 2^31 nodes: 140 bytes each at the least)
+__device__ __forceinline__ uint32_t cg_wrap_index(const CgGeom& g, int x, int y, int z) {
   x = x < 0 ? x + g.nx : (x >= g.nx ? x - g.nx : x);
   y = y < 0 ? y + g.ny : (y >= g.ny ? y - g.ny : y);
   z = z < 0 ? z + g.nz : (z >= g.nz ? z - g.nz : z);
-  return x + int64_t(g.nx) * (y + int64_t(g.ny) * z);
+  return uint32_t(x) + uint32_t(g.nx) * (uint32_t(y) + uint32_t(g.ny) * uint32_t(z));
 }
 
 // perturbation weights B_a by |c|^2 shell; sum B = cs2, sum B c c = cs2 I
@@ -68,146 +124,204 @@ __host__ __device__ constexpr double cg_B(int a) {
   return c2 == 0 ? -2.0 / 9.0 : (c2 == 1 ? 1.0 / 54.0 : 1.0 / 27.0);
 }
 
+// relaxation coefficients k of a node and c_R, c_RB <-> quads
+template <class L, class R>
+__device__ __forceinline__ void cg_store_coef(const CgSet<R>& s, int64_t n, uint32_t i, Coef<R>& k, R cr, R crb) {
+  constexpr int NC = n_coef<L>();
+  Quad<R> q[(NC + 2) / 4];
+  each_coef<L, R>(k, [&](auto I, R& v) { q[decltype(I)::value / 4].v[decltype(I)::value % 4] = v; });
+  q[NC / 4].v[NC % 4] = cr;
+  q[(NC + 1) / 4].v[(NC + 1) % 4] = crb;
+#pragma unroll
+  for (int j = 0; j < (NC + 2) / 4; ++j) s.k[j * n + i] = q[j];
+}
+
+// moment fields of a node from its populations' sums: g (all directions) and
+// the two colours' densities, shifted
+template <class L, class R>
+__device__ __forceinline__ void cg_store_moments(const CgSet<R>& s, int64_t n, uint32_t i, const R (&gt)[L::Q], R sr,
+                                                 R sb, const Phys<R>& ph, R half_rho0, R beta) {
+  Mom<R> m;
+  moments<L, R, false>(gt, ph, m);
+  Coef<R> k;
+  coeffs<L, R, false>(m, ph, k);
+  const R rr = sr + half_rho0, rb = sb + half_rho0, rho = rr + rb;
+  cg_store_coef<L>(s, n, i, k, rr / rho, beta * rr * rb / rho);
+  s.phi[i] = (rr - rb) / rho;
+}
+
+// constants of the pull
+template <class R>
+struct CgPull {
+  R pert_k, half_rho0;  // (9/4) sigma omega, rho0 / 2
+};
+
+// the populations that arrive at node (x, y, z): f(a, f_R, f_B), shifted
+template <class L, class R, class F>
+__device__ __forceinline__ void cg_pull(const CgGeom& g, const CgSet<R>& s, int x, int y, int z, const CgPull<R>& pc,
+                                        F&& f) {
+  constexpr int NC = n_coef<L>();
+  static_for<0, L::Q>([&](auto A_) {
+    constexpr int a = decltype(A_)::value;
+    constexpr int cx = L::cx(a), cy = L::cy(a), cz = L::cz(a);
+    const uint32_t u = cg_wrap_index(g, x - cx, y - cy, z - cz);  // upstream node
+    Quad<R> q[(NC + 2) / 4];
+#pragma unroll
+    for (int j = 0; j < (NC + 2) / 4; ++j) q[j] = s.k[j * g.n + u];
+    const Quad<R> gq = s.grad[u];
+    Coef<R> k{};
+    each_coef<L, R>(k, [&](auto I, R& v) { v = q[decltype(I)::value / 4].v[decltype(I)::value % 4]; });
+    const R cr = q[NC / 4].v[NC % 4], crb = q[(NC + 1) / 4].v[(NC + 1) % 4];
+    constexpr R w = R(weight<L>(a));
+    const R gpost = post<L, R, a>(k) + w * (R(2) * pc.half_rho0);  // unshifted relaxed total population
+    const R gn = gq.v[0];
+    R cn = R(0);  // c_a . n
+    if constexpr (cx != 0) cn = fma_r(R(cx), gq.v[1], cn);
+    if constexpr (cy != 0) cn = fma_r(R(cy), gq.v[2], cn);
+    if constexpr (cz != 0) cn = fma_r(R(cz), gq.v[3], cn);
+    constexpr R B = R(cg_B<L>(a));
+    const R gstar = fma_r(pc.pert_k * gn, fma_r(w * cn, cn, -B), gpost);
+    constexpr int c2 = cx * cx + cy * cy + cz * cz;
+    constexpr R inv_len = c2 == 0 ? R(0) : (c2 == 1 ? R(1) : (c2 == 2 ? R(0.70710678118654752440) :
+                                                                   R(0.57735026918962576451)));
+    const R rec = crb * (w * (cn * inv_len));
+    const R fred = fma_r(cr, gstar, rec);
+    const R fblue = gstar - fred;
+    f(A_, fred - w * pc.half_rho0, fblue - w * pc.half_rho0);
+  });
+}
+
 template <class L, class S, class R>
-__global__ void __launch_bounds__(kCgThreads) cg_moments_kernel(CgGeom g, const S* __restrict__ fr,
-                                                                  const S* __restrict__ fb, Phys<R> ph, R half_rho0,
-                                                                  R beta, R* __restrict__ fld) {
-  for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < g.n; i += int64_t(gridDim.x) * blockDim.x) {
-    R gt[L::Q];
-    R sr = R(0), sb = R(0);
-    static_for<0, L::Q>([&](auto A_) {
-      constexpr int a = decltype(A_)::value;
-      const R r = load_as<S, R>(fr[a * g.n + i]), b = load_as<S, R>(fb[a * g.n + i]);
-      sr = sr + r;
-      sb = sb + b;
-      gt[a] = r + b;
-    });
-    Mom<R> m;
-    moments<L, R, false>(gt, ph, m);
-    Coef<R> k;
-    coeffs<L, R, false>(m, ph, k);
-    fld[(F_COEF + 0) * g.n + i] = k.A;
-    for (int al = 0; al < 3; ++al) {
-      fld[(F_COEF + 1 + al) * g.n + i] = k.B[al];
-      fld[(F_COEF + 4 + al) * g.n + i] = k.C[al];
-      fld[(F_COEF + 7 + al) * g.n + i] = k.C2[al];
-    }
-    const R rr = sr + half_rho0, rb = sb + half_rho0, rho = rr + rb;
-    fld[F_CR * g.n + i] = rr / rho;
-    fld[F_CRB * g.n + i] = beta * rr * rb / rho;
-    fld[F_PHI * g.n + i] = (rr - rb) / rho;
-  }
+__global__ void __launch_bounds__(kCgThreads) cg_enter_kernel(const CgGeom g, const S* __restrict__ fr,
+                                                              const S* __restrict__ fb, const Phys<R> ph,
+                                                              R half_rho0, R beta, const CgSet<R> dst) {
+  const CgNode o = cg_node(g);
+  if (!o.in) return;
+  const uint32_t i = cg_wrap_index(g, o.x, o.y, o.z);
+  R gt[L::Q];
+  R sr = R(0), sb = R(0);
+  static_for<0, L::Q>([&](auto A_) {
+    constexpr int a = decltype(A_)::value;
+    const R r = load_as<S, R>(fr[a * g.n + i]), b = load_as<S, R>(fb[a * g.n + i]);
+    sr = sr + r;
+    sb = sb + b;
+    gt[a] = r + b;
+  });
+  cg_store_moments<L>(dst, g.n, i, gt, sr, sb, ph, half_rho0, beta);
+}
+
+// One step between sets.  Bound by the L1's vector loads and instruction issue
+// (a node pulls 9 or 19 directions of 48 or 64 bytes, DRAM sees each set once).
+template <class L, class S, class R>
+__global__ void __launch_bounds__(kCgThreads) cg_step_kernel(const CgGeom g, const CgSet<R> src, const Phys<R> ph,
+                                                             const CgPull<R> pc, R beta, const CgSet<R> dst) {
+  const CgNode o = cg_node(g);
+  if (!o.in) return;
+  R gt[L::Q];
+  R sr = R(0), sb = R(0);
+  cg_pull<L>(g, src, o.x, o.y, o.z, pc, [&](auto A_, R fr, R fb) {
+    const R r = round_to_storage<S, R>(fr), b = round_to_storage<S, R>(fb);
+    sr = sr + r;
+    sb = sb + b;
+    gt[decltype(A_)::value] = r + b;
+  });
+  cg_store_moments<L>(dst, g.n, cg_wrap_index(g, o.x, o.y, o.z), gt, sr, sb, ph, pc.half_rho0, beta);
+}
+
+template <class L, class S, class R>
+__global__ void __launch_bounds__(kCgThreads) cg_leave_kernel(const CgGeom g, const CgSet<R> src, const CgPull<R> pc,
+                                                              S* __restrict__ fr, S* __restrict__ fb) {
+  const CgNode o = cg_node(g);
+  if (!o.in) return;
+  const uint32_t i = cg_wrap_index(g, o.x, o.y, o.z);
+  cg_pull<L>(g, src, o.x, o.y, o.z, pc, [&](auto A_, R r, R b) {
+    constexpr int a = decltype(A_)::value;
+    fr[a * g.n + i] = store_as<S, R>(r);
+    fb[a * g.n + i] = store_as<S, R>(b);
+  });
 }
 
 // near-contact parameters of the gradient launch
 template <class R>
 struct CgNci {
-  R amp, bulk, half_rho0;  // A, -1 + eps, rho0 / 2
+  R amp, bulk;  // A, -1 + eps
   int h;
 };
 
-template <class L, class S, class R, bool NCI>
-__global__ void __launch_bounds__(kCgThreads) cg_gradient_kernel(CgGeom g, R* __restrict__ fld,
-                                                                  const S* __restrict__ fr,
-                                                                  const S* __restrict__ fb, Phys<R> ph,
-                                                                  CgNci<R> nci) {
-  const R* phi = fld + F_PHI * g.n;
-  for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < g.n; i += int64_t(gridDim.x) * blockDim.x) {
-    const int x = int(i % g.nx), y = int((i / g.nx) % g.ny), z = int(i / (int64_t(g.nx) * g.ny));
-    R gv[3] = {R(0), R(0), R(0)};
-    static_for<1, L::Q>([&](auto A_) {
-      constexpr int a = decltype(A_)::value;
-      const R p = phi[cg_wrap_index(g, x + L::cx(a), y + L::cy(a), z + L::cz(a))];
-      constexpr R w = R(weight<L>(a));
-      if constexpr (L::cx(a) != 0) gv[0] = fma_r(R(L::cx(a)) * w, p, gv[0]);
-      if constexpr (L::cy(a) != 0) gv[1] = fma_r(R(L::cy(a)) * w, p, gv[1]);
-      if constexpr (L::cz(a) != 0) gv[2] = fma_r(R(L::cz(a)) * w, p, gv[2]);
-    });
-    R g2 = R(0);
-    for (int al = 0; al < 3; ++al) {
-      gv[al] = gv[al] * R(3);  // 1 / cs2
-      g2 = fma_r(gv[al], gv[al], g2);
+// gradient of set s; prev: the set that s was stepped from (PULL), else its
+// populations are in fr, fb
+template <class L, class S, class R, bool NCI, bool PULL>
+__global__ void __launch_bounds__(kCgThreads) cg_gradient_kernel(const CgGeom g, const CgSet<R> s, const CgSet<R> prev,
+                                                                  const S* fr, const S* fb, const Phys<R> ph,
+                                                                  const CgPull<R> pc, const CgNci<R> nci) {
+  const CgNode o = cg_node(g);
+  if (!o.in) return;
+  const int x = o.x, y = o.y, z = o.z;
+  const uint32_t i = cg_wrap_index(g, x, y, z);
+  R gv[3] = {R(0), R(0), R(0)};
+  static_for<1, L::Q>([&](auto A_) {
+    constexpr int a = decltype(A_)::value;
+    const R p = s.phi[cg_wrap_index(g, x + L::cx(a), y + L::cy(a), z + L::cz(a))];
+    constexpr R w = R(weight<L>(a));
+    if constexpr (L::cx(a) != 0) gv[0] = fma_r(R(L::cx(a)) * w, p, gv[0]);
+    if constexpr (L::cy(a) != 0) gv[1] = fma_r(R(L::cy(a)) * w, p, gv[1]);
+    if constexpr (L::cz(a) != 0) gv[2] = fma_r(R(L::cz(a)) * w, p, gv[2]);
+  });
+  R g2 = R(0);
+  for (int al = 0; al < 3; ++al) {
+    gv[al] = gv[al] * R(3);  // 1 / cs2
+    g2 = fma_r(gv[al], gv[al], g2);
+  }
+  const R gn = sqrt(g2);
+  Quad<R> gq;
+  gq.v[0] = gn;
+  for (int al = 0; al < 3; ++al) gq.v[1 + al] = gn > R(0) ? gv[al] / gn : R(0);
+  s.grad[i] = gq;
+  if constexpr (NCI) {
+    bool flag = false;
+    if (s.phi[i] > nci.bulk && gn > R(0)) {
+      const int h = nci.h;
+      static_for<1, L::Q>([&](auto A_) {
+        constexpr int a = decltype(A_)::value;
+        constexpr int cx = L::cx(a), cy = L::cy(a), cz = L::cz(a);
+        const R p1 = s.phi[cg_wrap_index(g, x - h * cx, y - h * cy, z - h * cz)];
+        const R p2 = s.phi[cg_wrap_index(g, x - 2 * h * cx, y - 2 * h * cy, z - 2 * h * cz)];
+        flag = flag || (p1 < nci.bulk && p2 > nci.bulk);
+      });
     }
-    const R gn = sqrt(g2);
-    fld[F_GN * g.n + i] = gn;
-    for (int al = 0; al < 3; ++al) fld[(F_N + al) * g.n + i] = gn > R(0) ? gv[al] / gn : R(0);
-    if constexpr (NCI) {
-      bool flag = false;
-      if (phi[i] > nci.bulk) {
-        const int h = nci.h;
-        static_for<1, L::Q>([&](auto A_) {
-          constexpr int a = decltype(A_)::value;
-          constexpr int cx = L::cx(a), cy = L::cy(a), cz = L::cz(a);
-          const R p1 = phi[cg_wrap_index(g, x - h * cx, y - h * cy, z - h * cz)];
-          const R p2 = phi[cg_wrap_index(g, x - 2 * h * cx, y - 2 * h * cy, z - 2 * h * cz)];
-          flag = flag || (p1 < nci.bulk && p2 > nci.bulk);
+    if (flag) {
+      R gt[L::Q];
+      R sr = R(0);
+      if constexpr (PULL) {
+        cg_pull<L>(g, prev, x, y, z, pc, [&](auto A_, R r0, R b0) {
+          const R r = round_to_storage<S, R>(r0), b = round_to_storage<S, R>(b0);
+          sr = sr + r;
+          gt[decltype(A_)::value] = r + b;
         });
-      }
-      if (flag && gn > R(0)) {
-        R gt[L::Q];
-        R sr = R(0);
+      } else {
         static_for<0, L::Q>([&](auto A_) {
           constexpr int a = decltype(A_)::value;
           const R r = load_as<S, R>(fr[a * g.n + i]), b = load_as<S, R>(fb[a * g.n + i]);
           sr = sr + r;
           gt[a] = r + b;
         });
-        const R rr = sr + nci.half_rho0;  // rho_R
-        Phys<R> pf = ph;
-        for (int al = 0; al < 3; ++al) {
-          pf.F[al] = nci.amp * rr * (gv[al] / gn);
-          pf.hF[al] = R(0.5) * pf.F[al];
-        }
-        Mom<R> m;
-        moments<L, R, true>(gt, pf, m);
-        Coef<R> k;
-        coeffs<L, R, true>(m, pf, k);
-        fld[(F_COEF + 0) * g.n + i] = k.A;
-        for (int al = 0; al < 3; ++al) {
-          fld[(F_COEF + 1 + al) * g.n + i] = k.B[al];
-          fld[(F_COEF + 4 + al) * g.n + i] = k.C[al];
-          fld[(F_COEF + 7 + al) * g.n + i] = k.C2[al];
-        }
       }
-    }
-  }
-}
-
-template <class L, class S, class R>
-__global__ void __launch_bounds__(kCgThreads) cg_rebuild_kernel(CgGeom g, const R* __restrict__ fld, R pert_k,
-                                                                 R half_rho0, S* __restrict__ fr,
-                                                                 S* __restrict__ fb) {
-  for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < g.n; i += int64_t(gridDim.x) * blockDim.x) {
-    const int x = int(i % g.nx), y = int((i / g.nx) % g.ny), z = int(i / (int64_t(g.nx) * g.ny));
-    static_for<0, L::Q>([&](auto A_) {
-      constexpr int a = decltype(A_)::value;
-      constexpr int cx = L::cx(a), cy = L::cy(a), cz = L::cz(a);
-      const int64_t s = cg_wrap_index(g, x - cx, y - cy, z - cz);  // upstream node
-      Coef<R> k;
-      k.A = fld[(F_COEF + 0) * g.n + s];
+      const R rr = sr + pc.half_rho0;  // rho_R
+      Phys<R> pf = ph;
       for (int al = 0; al < 3; ++al) {
-        k.B[al] = fld[(F_COEF + 1 + al) * g.n + s];
-        k.C[al] = fld[(F_COEF + 4 + al) * g.n + s];
-        k.C2[al] = fld[(F_COEF + 7 + al) * g.n + s];
+        pf.F[al] = nci.amp * rr * gq.v[1 + al];
+        pf.hF[al] = R(0.5) * pf.F[al];
       }
-      constexpr R w = R(weight<L>(a));
-      const R gpost = post<L, R, a>(k) + w * (R(2) * half_rho0);  // unshifted relaxed total population
-      const R gn = fld[F_GN * g.n + s];
-      R cn = R(0);  // c_a . n
-      if constexpr (cx != 0) cn = fma_r(R(cx), fld[(F_N + 0) * g.n + s], cn);
-      if constexpr (cy != 0) cn = fma_r(R(cy), fld[(F_N + 1) * g.n + s], cn);
-      if constexpr (cz != 0) cn = fma_r(R(cz), fld[(F_N + 2) * g.n + s], cn);
-      constexpr R B = R(cg_B<L>(a));
-      const R gstar = fma_r(pert_k * gn, fma_r(w * cn, cn, -B), gpost);
-      constexpr int c2 = cx * cx + cy * cy + cz * cz;
-      constexpr R inv_len = c2 == 0 ? R(0) : (c2 == 1 ? R(1) : (c2 == 2 ? R(0.70710678118654752440) :
-                                                                     R(0.57735026918962576451)));
-      const R rec = fld[F_CRB * g.n + s] * (w * (cn * inv_len));
-      const R fred = fma_r(fld[F_CR * g.n + s], gstar, rec);
-      const R fblue = gstar - fred;
-      fr[a * g.n + i] = store_as<S, R>(fred - w * half_rho0);
-      fb[a * g.n + i] = store_as<S, R>(fblue - w * half_rho0);
-    });
+      Mom<R> m;
+      moments<L, R, true>(gt, pf, m);
+      Coef<R> k;
+      coeffs<L, R, true>(m, pf, k);
+      // the last quad keeps its c_R and c_RB
+      constexpr int NC = n_coef<L>(), last = NC / 4;
+      static_assert(NC % 4 == 2, "c_R and c_RB fill the last quad");
+      const Quad<R> q = s.k[last * g.n + i];
+      cg_store_coef<L>(s, g.n, i, k, q.v[2], q.v[3]);
+    }
   }
 }
 
@@ -289,16 +403,42 @@ int grid_of(int64_t n) {
   return int(b < 152 * 16 ? (b < 1 ? 1 : b) : 152 * 16);
 }
 
+// The box of a thread block: the power-of-two extents whose boxes cover the
+// domain with the fewest nodes, counting a third of the ring of neighbours that
+// a box reads (most of it from the L2 cache) and rows shorter than 4 nodes as
+// the sectors they half use.
+void plan_boxes(CgGeom& g) {
+  double best = 1e300;
+  for (int lx = 0; lx <= 8; ++lx)
+    for (int ly = 0; lx + ly <= 8; ++ly) {
+      const int lz = 8 - lx - ly;
+      const double bx = 1 << lx, by = 1 << ly, bz = 1 << lz;
+      const double tx = std::ceil(g.nx / bx), ty = std::ceil(g.ny / by), tz = std::ceil(g.nz / bz);
+      const double ring = (1 + 2 / bx) * (g.ny > 1 ? 1 + 2 / by : 1) * (1 + 2 / bz) - 1;
+      const double cost = tx * ty * tz * (1 + ring / 3) * (lx < 2 ? 2.0 : 1.0);
+      if (cost < best * (1 - 1e-9)) {
+        best = cost;
+        g.lx = lx;
+        g.ly = ly;
+        g.lz = lz;
+        g.ntx = uint32_t(tx);
+        g.nty = uint32_t(ty);
+        g.ntz = uint32_t(tz);
+      }
+    }
+}
+
 int rc_of(cudaError_t e) { return e == cudaSuccess ? LB_OK : (e == cudaErrorMemoryAllocation ? LB_E_NOMEM : LB_E_CUDA); }
 
 template <class F>
 bool cg_dispatch(int lattice, int storage, F&& f) {
-  if (lattice != LB_D2Q9 && lattice != LB_D3Q19) return false;
   if (storage != LB_F64 && storage != LB_F32) return false;
-  return dispatch_lattice(lattice, [&](auto Lt) {
+  auto on = [&](auto Lt) {
     if (storage == LB_F64) f(Lt, type_tag<double>{}, type_tag<double>{});
     else f(Lt, type_tag<float>{}, type_tag<float>{});
-  });
+    return true;
+  };
+  return lattice == LB_D2Q9 ? on(D2Q9{}) : lattice == LB_D3Q19 ? on(D3Q19{}) : false;
 }
 
 }  // namespace
@@ -378,6 +518,7 @@ int lb_cg_create(int32_t lattice, const int64_t dims[3], double tau, double sigm
   c->g.ny = d == 2 ? 1 : int(dims[1]);
   c->g.nz = d == 2 ? int(dims[1]) : int(dims[2]);
   c->g.n = dims[0] * dims[1] * dims[2];
+  plan_boxes(c->g);
   c->tau = tau;
   c->sigma = sigma;
   c->beta = beta;
@@ -499,28 +640,51 @@ int lb_cg_step(lb_cg* c, int64_t n) {
   Geometry geo{};
   geo.tau = c->tau;
   geo.rho0 = c->rho0;
-  bool ok = true;
-  for (int64_t s = 0; s < n && ok; ++s) {
-    ok = cg_dispatch(c->lattice, c->storage, [&](auto Lt, auto St, auto Rt) {
+  // runs of an odd number of steps end in set A; an even n takes one step first
+  while (n > 0) {
+    const int64_t run = n % 2 ? n : 1;
+    cg_dispatch(c->lattice, c->storage, [&](auto Lt, auto St, auto Rt) {
       using L = decltype(Lt);
       using S = typename decltype(St)::type;
       using R = typename decltype(Rt)::type;
       const Phys<R> ph = make_phys<R>(geo);
+      const CgPull<R> pc{R(2.25 * c->sigma / c->tau), R(0.5 * c->rho0)};
+      const CgNci<R> nci{R(c->nci_amp), R(-1.0 + c->nci_eps), c->nci_h};
+      S* fr = static_cast<S*>(c->fr);
+      S* fb = static_cast<S*>(c->fb);
+      // set A in fld; set B: the coefficients in f_R's array, the rest in f_B's
+      // (NC + 2 <= q and 4 + 1 <= q values a node)
+      static_assert(n_coef<L>() + 2 <= L::Q && 5 <= L::Q, "set B fits the population arrays");
       R* fld = static_cast<R*>(c->fld);
-      const int grid = grid_of(c->g.n);
-      cg_moments_kernel<L, S, R><<<grid, kCgThreads, 0, c->stream>>>(
-          c->g, static_cast<const S*>(c->fr), static_cast<const S*>(c->fb), ph, R(0.5 * c->rho0), R(c->beta), fld);
-      const CgNci<R> nci{R(c->nci_amp), R(-1.0 + c->nci_eps), R(0.5 * c->rho0), c->nci_h};
-      if (c->nci_amp != 0.0)
-        cg_gradient_kernel<L, S, R, true><<<grid, kCgThreads, 0, c->stream>>>(
-            c->g, fld, static_cast<const S*>(c->fr), static_cast<const S*>(c->fb), ph, nci);
-      else
-        cg_gradient_kernel<L, S, R, false><<<grid, kCgThreads, 0, c->stream>>>(c->g, fld, nullptr, nullptr, ph, nci);
-      cg_rebuild_kernel<L, S, R><<<grid, kCgThreads, 0, c->stream>>>(
-          c->g, fld, R(2.25 * c->sigma / c->tau), R(0.5 * c->rho0), static_cast<S*>(c->fr), static_cast<S*>(c->fb));
+      const int64_t N = c->g.n;
+      constexpr int NK = n_coef<L>() + 2;
+      auto quads = [](R* p) { return reinterpret_cast<Quad<R>*>(p); };
+      const CgSet<R> set[2] = {{quads(fld), quads(fld + NK * N), fld + (NK + 4) * N},
+                               {quads(reinterpret_cast<R*>(fr)), quads(reinterpret_cast<R*>(fb)),
+                                reinterpret_cast<R*>(fb) + 4 * N}};
+      const unsigned grid = c->g.ntx * c->g.nty * c->g.ntz;
+      auto gradient = [&](int which, auto pull) {
+        constexpr bool P = decltype(pull)::value;
+        if (c->nci_amp != 0.0)
+          cg_gradient_kernel<L, S, R, true, P><<<grid, kCgThreads, 0, c->stream>>>(c->g, set[which], set[1 - which], fr,
+                                                                                   fb, ph, pc, nci);
+        else
+          cg_gradient_kernel<L, S, R, false, false><<<grid, kCgThreads, 0, c->stream>>>(
+              c->g, set[which], set[1 - which], fr, fb, ph, pc, nci);
+      };
+      cg_enter_kernel<L, S, R>
+          <<<grid, kCgThreads, 0, c->stream>>>(c->g, fr, fb, ph, pc.half_rho0, R(c->beta), set[0]);
+      gradient(0, std::false_type{});
+      for (int64_t k = 1; k < run; ++k) {
+        const int src = int(k - 1) & 1;
+        cg_step_kernel<L, S, R><<<grid, kCgThreads, 0, c->stream>>>(c->g, set[src], ph, pc, R(c->beta), set[1 - src]);
+        gradient(1 - src, std::true_type{});
+      }
+      cg_leave_kernel<L, S, R><<<grid, kCgThreads, 0, c->stream>>>(c->g, set[0], pc, fr, fb);
     });
     if (cudaGetLastError() != cudaSuccess) return LB_E_CUDA;
-    c->steps_done++;
+    c->steps_done += run;
+    n -= run;
   }
   return LB_OK;
 }
