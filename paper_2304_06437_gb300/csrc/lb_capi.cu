@@ -461,8 +461,18 @@ int lb_create(int32_t lattice, const int64_t dims[3], double tau, const lb_bound
     const size_t aux_at = align256(ctx->f_bytes);
     size_t want = aux_at + ctx->aux_bytes;
     const size_t least = want;
-    if (ctx->scheme == LB_SCHEME_FUSED && !g.zlink[0] && !g.zlink[1])
-      want = std::max(want, moment_scratch_elems(g, ctx->storage) * ctx->real_bytes);
+    if (ctx->scheme == LB_SCHEME_FUSED && !g.zlink[0] && !g.zlink[1]) {
+      const size_t runs = std::max(moment_scratch_elems(g, ctx->storage), flat_scratch_elems(g, ctx->storage)) *
+                          ctx->real_bytes;
+      // the runs of 2D domains need much more than the
+      // populations: only where that is little of what is free, so that large
+      // domains, and many of them, still fit the card
+      size_t free_bytes = 0, total = 0;
+      const bool large = g.d == 2;
+      if (runs > want && (!large || (cudaMemGetInfo(&free_bytes, &total) == cudaSuccess && free_bytes > want &&
+                                     (free_bytes - want) / 16 >= runs - want)))
+        want = runs;
+    }
     cudaError_t e = cudaMalloc(&ctx->f, want);
     if (e == cudaErrorMemoryAllocation && want > least) {
       cudaGetLastError();
@@ -691,6 +701,11 @@ int lb_step(lb_ctx* ctx, int64_t n) {
   int64_t i = 0;
   if (n >= kMomentMinSteps && moment_plan(ctx)) {
     const cudaError_t e = moment_run(ctx, n);
+    if (e == cudaSuccess) ctx->steps_done += n;
+    return cuda_status(e);
+  }
+  if (n >= kMomentMinSteps && flat_plan(ctx)) {
+    const cudaError_t e = flat_run(ctx, n);
     if (e == cudaSuccess) ctx->steps_done += n;
     return cuda_status(e);
   }

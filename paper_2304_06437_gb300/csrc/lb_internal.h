@@ -100,6 +100,7 @@ struct lb_ctx {
   cudaGraphExec_t step_graph = nullptr;
   int graph_parity = 0;
   lbgb::MomentRun mr;
+  int flat_state = 0;     // runs of 2D domains: 0 not planned yet, 1 usable, -1 not
 };
 
 namespace lbgb {
@@ -149,6 +150,15 @@ void drop_moment_run(lb_ctx* ctx);
 // TMA descriptor of nf fields of the arithmetic type at base, boxes of bx x by
 // x 1 x nf (lb_capi.cu)
 bool make_field_map(lb_ctx* ctx, CUtensorMap* map, void* base, int nf, int bx, int by);
+
+// ---- runs of several steps of 2D domains (lb_k4.cu)
+// elements that the coefficient sets span from f on (0: none for this lattice
+// and storage)
+size_t flat_scratch_elems(const Geometry& g, int storage);
+// whether the context can run this way; plans it on the first call
+bool flat_plan(lb_ctx* ctx);
+// n >= 2 steps of a planned context
+cudaError_t flat_run(lb_ctx* ctx, int64_t n);
 
 // ---- state conversion, readout and reductions (lb_aux.cu)
 cudaError_t aux_set_populations(lb_ctx* ctx, const double* f_dev);

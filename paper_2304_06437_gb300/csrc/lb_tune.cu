@@ -55,6 +55,9 @@ int time_variant(const lb_ctx* ctx, const void* v, int steps, double* ns_per_upd
   int rc = lb_create(ctx->lattice, dims, ctx->tau_user, &ctx->bnd_user, &opt, &p);
   if (rc != LB_OK) return rc;
   rc = ctx_replan(p, v);
+  // runs on tiles of their own, from the first launch to the last, say nothing
+  // about the brick shape: time single steps
+  p->flat_state = -1;
   const double u[3] = {0.01, 0.005, 0.0};
   if (rc == LB_OK) rc = lb_init_uniform(p, ctx->g.rho0, u);
   cudaEvent_t e0 = nullptr, e1 = nullptr;
