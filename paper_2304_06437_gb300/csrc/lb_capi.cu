@@ -464,11 +464,11 @@ int lb_create(int32_t lattice, const int64_t dims[3], double tau, const lb_bound
     if (ctx->scheme == LB_SCHEME_FUSED && !g.zlink[0] && !g.zlink[1]) {
       const size_t runs = std::max(moment_scratch_elems(g, ctx->storage), flat_scratch_elems(g, ctx->storage)) *
                           ctx->real_bytes;
-      // the runs of 2D domains need much more than the
+      // the runs of 2D domains and of 16-bit ones need much more than the
       // populations: only where that is little of what is free, so that large
       // domains, and many of them, still fit the card
       size_t free_bytes = 0, total = 0;
-      const bool large = g.d == 2;
+      const bool large = g.d == 2 || ctx->elem_bytes == 2;
       if (runs > want && (!large || (cudaMemGetInfo(&free_bytes, &total) == cudaSuccess && free_bytes > want &&
                                      (free_bytes - want) / 16 >= runs - want)))
         want = runs;

@@ -132,11 +132,21 @@ cudaError_t k1_configure(lb_ctx* ctx);  // one-time kernel attributes
 // arithmetic-type elements that the two coefficient sets and their edge
 // records span from f on (0: no compiled tile for this lattice and storage)
 size_t moment_scratch_elems(const Geometry& g, int storage);
+// where set A (0) or B (1) of coefficient fields begins (lb_k3.cuh): A at the
+// populations' place and B behind it, or for 16-bit populations B at their
+// place and A behind both
+inline int64_t moment_set_at(const Geometry& g, int storage, int which) {
+  const int nc = g.d == 2 ? 6 : 10;
+  if (storage != LB_F16S && storage != LB_BF16S) return which ? nc * g.vol : 0;
+  const int pop = (g.q + 1) / 2;  // fields that the populations span
+  return which ? 0 : (pop > nc ? pop : nc) * g.vol;
+}
 // where the edge records begin: past both sets and past the populations (which
 // the conversion to set A or B still reads)
-inline int64_t moment_edge_at(const Geometry& g) {
-  const int sets = g.d == 2 ? 12 : 20;
-  return int64_t(g.q > sets ? g.q : sets) * g.vol;
+inline int64_t moment_edge_at(const Geometry& g, int storage) {
+  const int nc = g.d == 2 ? 6 : 10;
+  if (storage == LB_F16S || storage == LB_BF16S) return moment_set_at(g, storage, 0) + nc * g.vol;
+  return int64_t(g.q > 2 * nc ? g.q : 2 * nc) * g.vol;
 }
 // elements of one set's edge records for tiles bx wide
 inline int64_t moment_edge_elems(const Geometry& g, int bx) {

@@ -25,7 +25,8 @@
 // on one GB300, single-step launches against this form: D3Q19 FP32 512^3 35.2
 // -> 63.5 GLUPS (5.1 TB/s, 0.75 of the copy rate), 256^3 31.9 -> 60.3, 32^3
 // 24.8 -> 4.3 us; D3Q27 FP32 256^3 25.6 -> 47.0 (0.56); D3Q19 / D3Q27 FP64 96^3
-// 2.19 -> 3.17 / 1.10 -> 1.88 (bound by the FP64 rate).  What bounds the FP32
+// 2.19 -> 3.17 / 1.10 -> 1.88 (bound by the FP64 rate); D3Q19 FP16 160^3 161 ->
+// 72 us (57 GLUPS: the FP32 rate, two roundings a value on top).  What bounds the FP32
 // kernels: instruction issue (62 % of the slots) and, without the halo warps'
 // part, 71 GLUPS.
 //
@@ -33,7 +34,9 @@
 // itself -- set A in fields 0 .. n_coef - 1, set B in the n_coef fields after
 // it -- and its allocation goes on through the shell buffers (idle meanwhile,
 // rebuilt at the end), which hold what 2 n_coef fields exceed q by and the edge
-// records below.
+// records below.  16-bit populations are smaller than a set: set B takes their
+// place and what follows, set A the n_coef fields after that, and the last
+// step goes straight from set A to the populations (POP).
 //
 // Layout of a launch: a CTA owns a tile of bx x by nodes and sweeps bz planes.
 // TMA streams the tile's coefficients plane by plane into a ring of shared
@@ -77,6 +80,7 @@ struct K3Args {
   R* edst;
   int* status;
   uint32_t vol32;         // vol / 32 (rows are padded to 32 elements)
+  void* pop;              // populations written instead of dst (POP)
   R bb[27][8];
 };
 
@@ -160,8 +164,9 @@ LB_DEV R round_value(R v) { return round_to_storage<S, R>(v); }
 template <class S>
 LB_DEV f32x2 round_value(f32x2 v) { return round_pair<S>(v); }
 
-// One step of one brick (tile column tI, tJ, sweep tK): src -> dst.
-template <class L, class S, class R, int BX, int BY, int NS, int NPT, bool FORCE, int MINB>
+// One step of one brick (tile column tI, tJ, sweep tK): src -> dst, or (POP)
+// src -> populations, the last step of a run whose set A lies behind them.
+template <class L, class S, class R, int BX, int BY, int NS, int NPT, bool FORCE, int MINB, bool POP>
 __device__ __forceinline__ void k3_brick(
     const CUtensorMap* tmap_p, const K3Args<R, typename K3Shape<L, R, BX, BY, NS, NPT, MINB>::V>& args, const int tI,
     const int tJ, const int tK) {
@@ -572,29 +577,38 @@ __device__ __forceinline__ void k3_brick(
       // plane g - 1 is complete: collide it
       const int zd = g - 1;
       if (zd >= z0) {
-        V fr[Q];
-        static_for<0, Q>([&](auto A_) {
-          constexpr int a = decltype(A_)::value;
-          fr[a] = round_value<S>(G0[a]);
-        });
-        Coef<V> kc2;
-        moments_coeffs<L, FORCE>(fr, args.ph, kc2);
-        char* o = reinterpret_cast<char*>(out0 + plane * zd);
-        const uint32_t v32 = args.vol32;
-        if (NPT == 1 || act1) {
-          each_coef<L, V>(kc2, [&](auto I, V& v) {
-            *reinterpret_cast<V*>(o + uint64_t(v32) * uint32_t(decltype(I)::value * 32 * sizeof(R))) = v;
+        if constexpr (POP) {
+          static_assert(NPT == 1, "one node per thread");
+          S* o = static_cast<S*>(args.pop) + (x + args.pitch * y + plane * zd);
+          static_for<0, Q>([&](auto A_) {
+            constexpr int a = decltype(A_)::value;
+            o[a * args.vol] = store_as<S, R>(G0[a]);
           });
         } else {
-          each_coef<L, V>(kc2, [&](auto I, V& v) {
-            *reinterpret_cast<R*>(o + uint64_t(v32) * uint32_t(decltype(I)::value * 32 * sizeof(R))) = lane_of(v, 0);
+          V fr[Q];
+          static_for<0, Q>([&](auto A_) {
+            constexpr int a = decltype(A_)::value;
+            fr[a] = round_value<S>(G0[a]);
           });
-        }
-        if (west || east) {
-          R* e = edge0 + int64_t(ny) * NC * zd;
-          put_record<L>(kc2, e, west ? 0 : eastl);
-          // a tile of one column pair is both
-          if (west && east) put_record<L>(kc2, e + int64_t(args.ntx) * ny * nz * NC, eastl);
+          Coef<V> kc2;
+          moments_coeffs<L, FORCE>(fr, args.ph, kc2);
+          char* o = reinterpret_cast<char*>(out0 + plane * zd);
+          const uint32_t v32 = args.vol32;
+          if (NPT == 1 || act1) {
+            each_coef<L, V>(kc2, [&](auto I, V& v) {
+              *reinterpret_cast<V*>(o + uint64_t(v32) * uint32_t(decltype(I)::value * 32 * sizeof(R))) = v;
+            });
+          } else {
+            each_coef<L, V>(kc2, [&](auto I, V& v) {
+              *reinterpret_cast<R*>(o + uint64_t(v32) * uint32_t(decltype(I)::value * 32 * sizeof(R))) = lane_of(v, 0);
+            });
+          }
+          if (west || east) {
+            R* e = edge0 + int64_t(ny) * NC * zd;
+            put_record<L>(kc2, e, west ? 0 : eastl);
+            // a tile of one column pair is both
+            if (west && east) put_record<L>(kc2, e + int64_t(args.ntx) * ny * nz * NC, eastl);
+          }
         }
       }
     }
@@ -630,13 +644,13 @@ __device__ __forceinline__ void k3_brick(
   }
 }
 
-template <class L, class S, class R, int BX, int BY, int NS, int NPT, bool FORCE, int MINB>
+template <class L, class S, class R, int BX, int BY, int NS, int NPT, bool FORCE, int MINB, bool POP = false>
 __global__ void __launch_bounds__(K3Shape<L, R, BX, BY, NS, NPT, MINB>::NT, MINB)
     k3_step(const __grid_constant__ CUtensorMap tmap,
             const __grid_constant__ K3Args<R, typename K3Shape<L, R, BX, BY, NS, NPT, MINB>::V> args) {
   const int b = blockIdx.x;
-  k3_brick<L, S, R, BX, BY, NS, NPT, FORCE, MINB>(&tmap, args, b % args.ntx, (b / args.ntx) % args.nty,
-                                                  b / (args.ntx * args.nty));
+  k3_brick<L, S, R, BX, BY, NS, NPT, FORCE, MINB, POP>(&tmap, args, b % args.ntx, (b / args.ntx) % args.nty,
+                                                       b / (args.ntx * args.nty));
 }
 
 // Populations -> coefficient fields and edge records, node by node (each thread

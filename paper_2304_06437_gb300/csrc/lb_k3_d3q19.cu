@@ -9,6 +9,8 @@ extern const K3Variant k3_variants_d3q19[] = {
     K3Impl<D3Q19, float, float, 32, 16, 3, 1, 1>::variant(LB_D3Q19, LB_F32),
     K3Impl<D3Q19, float, float, 32, 4, 2, 1, 2>::variant(LB_D3Q19, LB_F32),  // small domains
     K3Impl<D3Q19, double, double, 32, 8, 2, 1, 1>::variant(LB_D3Q19, LB_F64),
+    K3Impl<D3Q19, __half, float, 32, 16, 3, 1, 1>::variant(LB_D3Q19, LB_F16S),
+    K3Impl<D3Q19, __nv_bfloat16, float, 32, 16, 3, 1, 1>::variant(LB_D3Q19, LB_BF16S),
 };
 extern const int k3_n_variants_d3q19 = sizeof(k3_variants_d3q19) / sizeof(k3_variants_d3q19[0]);
 

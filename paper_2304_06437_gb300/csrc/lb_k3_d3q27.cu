@@ -8,6 +8,8 @@ namespace lbgb {
 extern const K3Variant k3_variants_d3q27[] = {
     K3Impl<D3Q27, float, float, 32, 12, 3, 1, 1>::variant(LB_D3Q27, LB_F32),
     K3Impl<D3Q27, double, double, 32, 6, 2, 1, 1>::variant(LB_D3Q27, LB_F64),
+    K3Impl<D3Q27, __half, float, 32, 12, 3, 1, 1>::variant(LB_D3Q27, LB_F16S),
+    K3Impl<D3Q27, __nv_bfloat16, float, 32, 12, 3, 1, 1>::variant(LB_D3Q27, LB_BF16S),
 };
 extern const int k3_n_variants_d3q27 = sizeof(k3_variants_d3q27) / sizeof(k3_variants_d3q27[0]);
 

@@ -16,6 +16,8 @@ struct K3Variant {
   // one step of the context's domain: set src (0 = A, 1 = B) to the other
   cudaError_t (*step)(lb_ctx*, int src);
   cudaError_t (*enter)(lb_ctx*, int dst);  // populations -> coefficient set dst
+  // 16-bit storage: the last step, set A -> populations (else null, see LeaveVariant)
+  cudaError_t (*leave)(lb_ctx*);
 };
 
 // The launches that end a run for contexts whose brick cross-section is
@@ -28,13 +30,11 @@ struct LeaveVariant {
   cudaError_t (*leave)(lb_ctx*);
 };
 
-template <class L>
-LB_HD constexpr int coef_set_b() { return L::D == 2 ? 6 : 10; }
-
 template <class L, class S, class R, int BX, int BY, int NS, int NPT, int MINB>
 struct K3Impl {
   using Sh = K3Shape<L, R, BX, BY, NS, NPT, MINB>;
   using V = typename Sh::V;
+  static constexpr bool HALF = sizeof(S) == 2;
 
   static cudaError_t configure() {
     cudaError_t e = cudaFuncSetAttribute(k3_step<L, S, R, BX, BY, NS, NPT, false, MINB>,
@@ -42,19 +42,23 @@ struct K3Impl {
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(k3_step<L, S, R, BX, BY, NS, NPT, true, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                int(Sh::SMEM));
+    if constexpr (HALF)
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k3_step<L, S, R, BX, BY, NS, NPT, false, MINB, true>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, int(Sh::SMEM));
     return e;
   }
 
   static R* coef_set(lb_ctx* ctx, int which) {
-    return static_cast<R*>(ctx->f) + (which ? int64_t(coef_set_b<L>()) * ctx->g.vol : 0);
+    return static_cast<R*>(ctx->f) + moment_set_at(ctx->g, ctx->storage, which);
   }
 
   // the edge records of a set, after the two sets (moment_scratch_elems)
   static R* edges(lb_ctx* ctx, int which) {
-    return static_cast<R*>(ctx->f) + moment_edge_at(ctx->g) + which * moment_edge_elems(ctx->g, BX);
+    return static_cast<R*>(ctx->f) + moment_edge_at(ctx->g, ctx->storage) + which * moment_edge_elems(ctx->g, BX);
   }
 
-  static cudaError_t step(lb_ctx* ctx, int src) {
+  static K3Args<R, V> args_of(lb_ctx* ctx, int src) {
     const Geometry& g = ctx->g;
     K3Args<R, V> a;
     a.ph = make_phys<V>(g);
@@ -76,13 +80,29 @@ struct K3Impl {
     a.status = ctx->d_status;
     for (int i = 0; i < 27; ++i)
       for (int j = 0; j < 8; ++j) a.bb[i][j] = R(0);
+    a.pop = ctx->f;
     make_bounce_terms<L, R>(g, a.bb);
+    return a;
+  }
+
+  static cudaError_t step(lb_ctx* ctx, int src) {
+    const K3Args<R, V> a = args_of(ctx, src);
     const int grid = a.ntx * a.nty * a.ntz;
     const CUtensorMap& tm = ctx->mr.maps[src];
-    if (g.has_force)
+    if (ctx->g.has_force)
       k3_step<L, S, R, BX, BY, NS, NPT, true, MINB><<<grid, Sh::NT, Sh::SMEM, ctx->stream>>>(tm, a);
     else
       k3_step<L, S, R, BX, BY, NS, NPT, false, MINB><<<grid, Sh::NT, Sh::SMEM, ctx->stream>>>(tm, a);
+    return cudaGetLastError();
+  }
+
+  // (no collision: one instantiation serves with and without a force)
+  static cudaError_t leave(lb_ctx* ctx) {
+    if constexpr (HALF) {
+      const K3Args<R, V> a = args_of(ctx, 0);
+      k3_step<L, S, R, BX, BY, NS, NPT, false, MINB, true>
+          <<<a.ntx * a.nty * a.ntz, Sh::NT, Sh::SMEM, ctx->stream>>>(ctx->mr.maps[0], a);
+    }
     return cudaGetLastError();
   }
 
@@ -101,7 +121,7 @@ struct K3Impl {
   }
 
   static constexpr K3Variant variant(int lattice, int storage) {
-    return K3Variant{lattice, storage, BX, BY, NS, NPT, MINB, &configure, &step, &enter};
+    return K3Variant{lattice, storage, BX, BY, NS, NPT, MINB, &configure, &step, &enter, HALF ? &leave : nullptr};
   }
 };
 

@@ -67,7 +67,7 @@ int choose_bz(int nz, int64_t columns, int slots) {
 size_t moment_scratch_elems(const Geometry& g, int storage) {
   const K3Variant* v = find_k3(g, storage);
   if (!v) return 0;
-  return size_t(moment_edge_at(g)) + 2 * size_t(moment_edge_elems(g, v->bx));
+  return size_t(moment_edge_at(g, storage)) + 2 * size_t(moment_edge_elems(g, v->bx));
 }
 
 bool moment_plan(lb_ctx* ctx) {
@@ -77,18 +77,18 @@ bool moment_plan(lb_ctx* ctx) {
   if (ctx->scheme != LB_SCHEME_FUSED || ctx->g.zlink[0] || ctx->g.zlink[1]) return false;
   m.v = find_k3(ctx->g, ctx->storage);
   m.lv = find_leave(ctx->lattice, ctx->storage, ctx->plan.bx, ctx->plan.by);
-  if (!m.v || !m.lv) return false;
+  if (!m.v || (!m.lv && !m.v->leave)) return false;
   if (ctx->f_alloc < moment_scratch_elems(ctx->g, ctx->storage) * ctx->real_bytes) return false;
   const Geometry& g = ctx->g;
   m.bz = choose_bz(g.nz, int64_t(div_up(g.nx, m.v->bx)) * div_up(g.ny, m.v->by), k1_sm_count() * m.v->minb);
   const int nc = g.d == 2 ? 6 : 10;
-  bool ok = make_field_map(ctx, &m.tmap_leave, ctx->f, nc, m.lv->bx, m.lv->by);
+  bool ok = !m.lv || make_field_map(ctx, &m.tmap_leave, ctx->f, nc, m.lv->bx, m.lv->by);
   for (int set = 0; set < 2; ++set) {
-    void* base = static_cast<char*>(ctx->f) + size_t(set * nc) * size_t(g.vol) * ctx->real_bytes;
+    void* base = static_cast<char*>(ctx->f) + size_t(moment_set_at(g, ctx->storage, set)) * ctx->real_bytes;
     ok = ok && make_field_map(ctx, &m.maps[set], base, nc, m.v->bx, m.v->by);
   }
   if (!ok) return false;
-  if (m.v->configure() != cudaSuccess || m.lv->configure() != cudaSuccess) {
+  if (m.v->configure() != cudaSuccess || (m.lv && m.lv->configure() != cudaSuccess)) {
     cudaGetLastError();
     return false;
   }
@@ -125,10 +125,16 @@ bool capture_steps(lb_ctx* ctx) {
 
 cudaError_t moment_run(lb_ctx* ctx, int64_t n) {
   MomentRun& m = ctx->mr;
-  // the last step leaves from set A: an odd number of launches starts from B
+  // the last step leaves from set A: an odd number of launches starts from B,
+  // or, where the populations lie in set B's place, after a single step
+  cudaError_t e = cudaSuccess;
+  if (m.v->leave && n % 2 == 0) {
+    e = k1_step(ctx);
+    --n;
+  }
   const int64_t launches = n - 1;
   int src = int(launches & 1);
-  cudaError_t e = m.v->enter(ctx, src);
+  if (e == cudaSuccess) e = m.v->enter(ctx, src);
   int64_t i = 0;
   if (e == cudaSuccess && src) {
     e = m.v->step(ctx, 1);
@@ -141,6 +147,10 @@ cudaError_t moment_run(lb_ctx* ctx, int64_t n) {
     for (; i + kMomentGraphSteps <= launches && e == cudaSuccess; i += kMomentGraphSteps)
       e = cudaGraphLaunch(m.graph, ctx->stream);
   for (src = 0; i < launches && e == cudaSuccess; ++i, src = 1 - src) e = m.v->step(ctx, src);
+  if (m.v->leave) {
+    if (e == cudaSuccess) e = m.v->leave(ctx);
+    return e == cudaSuccess ? k1_bootstrap(ctx) : e;
+  }
   if (e == cudaSuccess) e = m.lv->shell(ctx);
   if (e == cudaSuccess) e = m.lv->leave(ctx);
   if (e == cudaSuccess) ctx->parity = 1 - ctx->parity;

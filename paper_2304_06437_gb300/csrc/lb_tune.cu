@@ -58,6 +58,7 @@ int time_variant(const lb_ctx* ctx, const void* v, int steps, double* ns_per_upd
   // runs on tiles of their own, from the first launch to the last, say nothing
   // about the brick shape: time single steps
   p->flat_state = -1;
+  if (p->elem_bytes == 2) p->mr.state = -1;
   const double u[3] = {0.01, 0.005, 0.0};
   if (rc == LB_OK) rc = lb_init_uniform(p, ctx->g.rho0, u);
   cudaEvent_t e0 = nullptr, e1 = nullptr;
