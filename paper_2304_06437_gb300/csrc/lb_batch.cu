@@ -10,6 +10,10 @@
 // launches of two consecutive steps of all classes are captured in a CUDA
 // graph and replayed, so a long run costs one graph launch per two steps.
 //
+// In calls of several steps, members of some size run one by one on a few
+// streams of the batch in moment form (lb_k3.cuh, lb_k4.cu), side by side and beside the classes of
+// the members that are left: a second list of classes and a second graph.
+//
 // The per-node arithmetic, the bricks and the shells are exactly those of
 // the domain's own single-domain launches: every domain's populations are bit
 // for bit those of stepping it alone.
@@ -39,13 +43,19 @@ struct lb_batch {
     int n_items = 0, grid = 0;
   };
   std::vector<Class> classes;
+  std::vector<int> runs;    // members that calls of several steps run on their own,
+  std::vector<int> lane;    // the stream (of lanes) that each of them runs on, and
+  std::vector<Class> rest;  // the classes of the others
   int* d_status = nullptr;
-  cudaGraphExec_t graph = nullptr;
+  cudaGraphExec_t graph = nullptr;       // two steps of all classes, and
+  cudaGraphExec_t rest_graph = nullptr;  // of the rest
   cudaEvent_t done = nullptr;
   cudaEvent_t fork = nullptr;          // class branches of one step
   std::vector<cudaStream_t> side;      // one per class after the first
   std::vector<cudaEvent_t> join;
   std::vector<cudaEvent_t> ctx_ev;
+  std::vector<cudaStream_t> lanes;
+  std::vector<cudaEvent_t> lane_ev;
   int64_t steps_done = 0;
   int64_t total_nodes = 0;
   double* d_sums = nullptr;  // lb_batch_reduce: seven sums per member (device)
@@ -245,17 +255,27 @@ int split_for_balance(lb_batch& b, lb_batch::Class& c) {
   return LB_OK;
 }
 
+// Whether calls of several steps run a member on its own.  A step of such a run
+// costs the host about a microsecond (a recorded graph of eight launches in
+// 3D, a launch for up to eight steps in 2D), which a member has to be worth on
+// the device; the classes carry the smaller ones at no cost of their own.
+bool runs_alone(lb_ctx* x) {
+  constexpr int64_t kMin3d = 65536, kMin2d = 16384;
+  if (x->n_nodes < (x->g.d == 2 ? kMin2d : kMin3d)) return false;
+  return moment_plan(x) || flat_plan(x);
+}
+
 // One step (k = 0 or 1 of the captured pair) of every class.  Classes are
 // independent domains: each runs on its own branch (the batch stream for the
 // first, a side stream forked from it for the others) and all join back.
-int launch_classes(lb_batch& b, int k) {
-  const int nc = int(b.classes.size());
+int launch_classes(lb_batch& b, std::vector<lb_batch::Class>& classes, int k) {
+  const int nc = int(classes.size());
   if (nc > 1) {
     LB_BTRY(cudaEventRecord(b.fork, b.stream));
     for (int i = 1; i < nc; ++i) LB_BTRY(cudaStreamWaitEvent(b.side[i - 1], b.fork, 0));
   }
   for (int i = 0; i < nc; ++i) {
-    auto& c = b.classes[i];
+    auto& c = classes[i];
     const BatchLaunch L{c.d_args, int(c.members.size()), c.d_tmaps, c.d_items, c.d_starts, c.d_par,
                         c.grid, k, c.force};
     LB_BTRY(c.v->batched(L, i == 0 ? b.stream : b.side[i - 1]));
@@ -268,8 +288,8 @@ int launch_classes(lb_batch& b, int k) {
 }
 
 // upload each member's current shell parity if it changed since the last step
-int sync_parities(lb_batch& b) {
-  for (auto& c : b.classes) {
+int sync_parities(lb_batch& b, std::vector<lb_batch::Class>& classes) {
+  for (auto& c : classes) {
     bool changed = false;
     for (size_t m = 0; m < c.members.size(); ++m) {
       const int p = b.ctxs[c.members[m]]->parity;
@@ -281,6 +301,34 @@ int sync_parities(lb_batch& b) {
     for (size_t m = 0; m < c.members.size(); ++m) c.h_par[m] = b.ctxs[c.members[m]]->parity;
     LB_BTRY(cudaMemcpyAsync(c.d_par, c.h_par, c.members.size() * sizeof(int), cudaMemcpyHostToDevice, b.stream));
   }
+  return LB_OK;
+}
+
+// two consecutive steps of the classes as a graph
+int capture_pair(lb_batch& b, std::vector<lb_batch::Class>& classes, cudaGraphExec_t* out) {
+  cudaGraph_t g = nullptr;
+  LB_BTRY(cudaStreamBeginCapture(b.stream, cudaStreamCaptureModeThreadLocal));
+  int rc = launch_classes(b, classes, 0);
+  if (rc == LB_OK) rc = launch_classes(b, classes, 1);
+  const cudaError_t e = cudaStreamEndCapture(b.stream, &g);
+  if (rc == LB_OK) rc = cuda_rc(e);
+  if (rc == LB_OK) rc = cuda_rc(cudaGraphInstantiate(out, g, 0));
+  if (g) cudaGraphDestroy(g);
+  return rc;
+}
+
+// n steps of the given classes on the batch stream
+int step_classes(lb_batch& b, std::vector<lb_batch::Class>& classes, cudaGraphExec_t graph, int64_t n) {
+  int rc = sync_parities(b, classes);
+  if (rc != LB_OK) return rc;
+  for (int64_t s = 0; s + 1 < n; s += 2) LB_BTRY(cudaGraphLaunch(graph, b.stream));
+  if (n & 1) rc = launch_classes(b, classes, 0);
+  if (rc != LB_OK) return rc;
+  for (auto& c : classes)
+    for (int m : c.members) {
+      if (n & 1) b.ctxs[m]->parity = 1 - b.ctxs[m]->parity;
+      b.ctxs[m]->steps_done += n;
+    }
   return LB_OK;
 }
 
@@ -368,20 +416,44 @@ int lb_batch_create(lb_ctx* const* ctxs, int32_t n, void* stream, lb_batch** out
     for (int i = 0; i < n && rc == LB_OK; ++i)
       if (cudaEventCreateWithFlags(&b->ctx_ev[i], cudaEventDisableTiming) != cudaSuccess) rc = LB_E_CUDA;
     if (rc != LB_OK) break;
-    // capture two consecutive steps of every class
-    cudaGraph_t g = nullptr;
-    if (cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) { rc = LB_E_CUDA; break; }
-    int rc0 = launch_classes(*b, 0);
-    int rc1 = rc0 == LB_OK ? launch_classes(*b, 1) : rc0;
-    cudaError_t ee = cudaStreamEndCapture(b->stream, &g);
-    if (rc1 != LB_OK || ee != cudaSuccess) {
-      if (g) cudaGraphDestroy(g);
-      rc = rc1 != LB_OK ? rc1 : LB_E_CUDA;
-      break;
+    if ((rc = capture_pair(*b, b->classes, &b->graph)) != LB_OK) break;
+    // members that run alone, the largest first, and the classes without them
+    for (int i = 0; i < n; ++i)
+      if (runs_alone(ctxs[i])) b->runs.push_back(i);
+    std::stable_sort(b->runs.begin(), b->runs.end(),
+                     [&](int i, int j) { return ctxs[i]->n_nodes > ctxs[j]->n_nodes; });
+    // (eight lanes: the streams that the device runs side by side by default),
+    // each to the least loaded
+    const size_t lanes = std::min<size_t>(b->runs.size(), 8);
+    std::vector<int64_t> load(lanes, 0);
+    for (int i : b->runs) {
+      const size_t k = std::min_element(load.begin(), load.end()) - load.begin();
+      b->lane.push_back(int(k));
+      load[k] += ctxs[i]->n_nodes;
     }
-    ee = cudaGraphInstantiate(&b->graph, g, 0);
-    cudaGraphDestroy(g);
-    if (ee != cudaSuccess) { rc = LB_E_CUDA; break; }
+    for (size_t k = 0; k < lanes && rc == LB_OK; ++k) {
+      cudaStream_t st = nullptr;
+      cudaEvent_t ev = nullptr;
+      rc = cuda_rc(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
+      if (rc == LB_OK) b->lanes.push_back(st);
+      if (rc == LB_OK) rc = cuda_rc(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+      if (rc == LB_OK) b->lane_ev.push_back(ev);
+    }
+    if (rc != LB_OK) break;
+    if (!b->runs.empty()) {
+      for (const auto& c : b->classes) {
+        lb_batch::Class r;
+        r.v = c.v;
+        r.force = c.force;
+        for (int m : c.members)
+          if (std::find(b->runs.begin(), b->runs.end(), m) == b->runs.end()) r.members.push_back(m);
+        if (r.members.empty()) continue;
+        b->rest.push_back(r);
+        if ((rc = setup_class(*b, b->rest.back())) != LB_OK) break;
+      }
+      if (rc == LB_OK && !b->rest.empty()) rc = capture_pair(*b, b->rest, &b->rest_graph);
+      if (rc != LB_OK) break;
+    }
     if (cudaStreamSynchronize(b->stream) != cudaSuccess) { rc = LB_E_CUDA; break; }
   } while (false);
   if (rc != LB_OK) {
@@ -401,17 +473,28 @@ int lb_batch_step(lb_batch* b, int64_t n) {
     LB_BTRY(cudaEventRecord(b->ctx_ev[i], b->ctxs[i]->stream));
     LB_BTRY(cudaStreamWaitEvent(b->stream, b->ctx_ev[i], 0));
   }
-  int rc = sync_parities(*b);
+  int rc = LB_OK;
+  if (n >= kMomentMinSteps && !b->runs.empty()) {
+    LB_BTRY(cudaEventRecord(b->done, b->stream));
+    for (cudaStream_t st : b->lanes) LB_BTRY(cudaStreamWaitEvent(st, b->done, 0));
+    for (size_t k = 0; k < b->runs.size() && rc == LB_OK; ++k) {
+      lb_ctx* x = b->ctxs[b->runs[k]];
+      // the launches of a run go to the stream of the context
+      const cudaStream_t own = x->stream;
+      x->stream = b->lanes[b->lane[k]];
+      rc = cuda_rc(moment_plan(x) ? moment_run(x, n) : flat_run(x, n));
+      x->stream = own;
+      x->steps_done += n;
+    }
+    if (rc == LB_OK && !b->rest.empty()) rc = step_classes(*b, b->rest, b->rest_graph, n);
+    for (size_t k = 0; k < b->lanes.size(); ++k) {
+      LB_BTRY(cudaEventRecord(b->lane_ev[k], b->lanes[k]));
+      LB_BTRY(cudaStreamWaitEvent(b->stream, b->lane_ev[k], 0));
+    }
+  } else {
+    rc = step_classes(*b, b->classes, b->graph, n);
+  }
   if (rc != LB_OK) return rc;
-  for (int64_t s = 0; s + 1 < n; s += 2) LB_BTRY(cudaGraphLaunch(b->graph, b->stream));
-  if (n & 1) {
-    rc = launch_classes(*b, 0);
-    if (rc != LB_OK) return rc;
-  }
-  for (lb_ctx* x : b->ctxs) {
-    if (n & 1) x->parity = 1 - x->parity;
-    x->steps_done += n;
-  }
   b->steps_done += n;
   // later work on a member's stream sees the batch's steps
   LB_BTRY(cudaEventRecord(b->done, b->stream));
@@ -424,7 +507,13 @@ int lb_batch_sync(lb_batch* b) {
   DevGuard guard(b->device);
   int st = 0;
   LB_BTRY(cudaMemcpyAsync(&st, b->d_status, sizeof(int), cudaMemcpyDeviceToHost, b->stream));
+  // members that ran alone report to their own status word
+  std::vector<int> own(b->runs.size(), 0);
+  for (size_t k = 0; k < own.size(); ++k)
+    LB_BTRY(cudaMemcpyAsync(&own[k], b->ctxs[b->runs[k]]->d_status, sizeof(int), cudaMemcpyDeviceToHost, b->stream));
   LB_BTRY(cudaStreamSynchronize(b->stream));
+  for (int v : own)
+    if (st == 0) st = v;
   return st != 0 ? st : LB_OK;
 }
 
@@ -484,7 +573,9 @@ void lb_batch_destroy(lb_batch* b) {
   DevGuard guard(b->device);
   if (b->stream) cudaStreamSynchronize(b->stream);
   if (b->graph) cudaGraphExecDestroy(b->graph);
+  if (b->rest_graph) cudaGraphExecDestroy(b->rest_graph);
   for (auto& c : b->classes) free_class(c);
+  for (auto& c : b->rest) free_class(c);
   if (b->d_status) cudaFree(b->d_status);
   if (b->done) cudaEventDestroy(b->done);
   if (b->fork) cudaEventDestroy(b->fork);
@@ -494,6 +585,8 @@ void lb_batch_destroy(lb_batch* b) {
     if (st) cudaStreamDestroy(st);
   for (cudaEvent_t e : b->ctx_ev)
     if (e) cudaEventDestroy(e);
+  for (cudaEvent_t e : b->lane_ev) cudaEventDestroy(e);
+  for (cudaStream_t st : b->lanes) cudaStreamDestroy(st);
   if (b->d_sums) cudaFree(b->d_sums);
   if (b->h_sums) cudaFreeHost(b->h_sums);
   if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
