@@ -318,6 +318,9 @@ LB_API int lb_autotune(lb_ctx* ctx, int32_t steps, lb_tune_entry* table, int32_t
  * sweeps of up to 256 planes; where a class would then have fewer than two
  * bricks per persistent CTA, its members' sweeps are halved (down to 64
  * planes) until it has.  Classes run on parallel branches of the graph.
+ * Calls of four or more steps take members of at least 65536 nodes (2D: 16384)
+ * through the runs that lb_step() has for several steps, on streams of the
+ * batch and beside the classes of the other members.
  * stream: cudaStream_t for the batch's work, NULL = a library-owned stream.
  * Errors: LB_E_INVAL (NULL, duplicates, mixed devices), LB_E_UNSUPPORTED,
  * LB_E_NOMEM, LB_E_CUDA. */
@@ -359,12 +362,12 @@ LB_API void lb_batch_destroy(lb_batch* b);
 
 /* --------------------------------------------------- two-component model
  * The paper's colour-gradient (CG) model for two immiscible fluids, red and
- * blue (section 2.1), in the thread-safe form of section 4: per step one
- * launch takes the moments of each node (the regularized relaxation
- * coefficients of the total set g = f_R + f_B, the concentrations and the
- * phase field phi = (rho_R - rho_B)/rho), one takes grad phi by the isotropic
- * stencil (1/cs2) sum_a t_a c_a phi(x + c_a), and one rebuilds both colours
- * at every node from the upstream node's fields:
+ * blue (section 2.1), in the thread-safe form of section 4: the moments of each
+ * node (the regularized relaxation coefficients of the total set g = f_R +
+ * f_B, the concentrations and the phase field phi = (rho_R - rho_B)/rho), then
+ * grad phi by the isotropic stencil (1/cs2) sum_a t_a c_a phi(x + c_a), then
+ * both colours at every node from the upstream nodes' fields (two launches a
+ * step; between the steps of one call the populations are not stored):
  *   g*_a = [Eq. LBexp with fhat^neq]_a + (9/4) sigma omega |grad phi|
  *          [t_a (c_a.n)^2 - B_a]                          (perturbation)
  *   f_R,a = (rho_R/rho) g*_a + beta (rho_R rho_B/rho) t_a (c_a.n)/|c_a|,
