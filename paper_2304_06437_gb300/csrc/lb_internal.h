@@ -54,6 +54,7 @@ struct MomentRun {
   const K3Variant* v = nullptr;
   const LeaveVariant* lv = nullptr;
   int bz = 0;
+  bool shared = false;  // beside other runs: launches keep no room for the next
   CUtensorMap maps[2];  // sets A and B, boxes of a tile
   CUtensorMap tmap_leave;
   cudaGraphExec_t graph = nullptr;
@@ -157,6 +158,9 @@ bool moment_plan(lb_ctx* ctx);
 // n >= 2 steps of a planned context
 cudaError_t moment_run(lb_ctx* ctx, int64_t n);
 void drop_moment_run(lb_ctx* ctx);
+// the run of a planned context beside others: recorded steps of its own, whose
+// launches keep no room for the next, for the context while it runs so
+MomentRun moment_plan_beside(const lb_ctx* ctx);
 // TMA descriptor of nf fields of the arithmetic type at base, boxes of bx x by
 // x 1 x nf (lb_capi.cu)
 bool make_field_map(lb_ctx* ctx, CUtensorMap* map, void* base, int nf, int bx, int by);
@@ -167,8 +171,8 @@ bool make_field_map(lb_ctx* ctx, CUtensorMap* map, void* base, int nf, int bx, i
 size_t flat_scratch_elems(const Geometry& g, int storage);
 // whether the context can run this way; plans it on the first call
 bool flat_plan(lb_ctx* ctx);
-// n >= 2 steps of a planned context
-cudaError_t flat_run(lb_ctx* ctx, int64_t n);
+// n >= 2 steps of a planned context; beside: other runs share the device
+cudaError_t flat_run(lb_ctx* ctx, int64_t n, bool beside = false);
 
 // ---- state conversion, readout and reductions (lb_aux.cu)
 cudaError_t aux_set_populations(lb_ctx* ctx, const double* f_dev);

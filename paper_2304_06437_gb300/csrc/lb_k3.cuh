@@ -215,8 +215,13 @@ __device__ __forceinline__ void k3_brick(
     for (int s = 0; s < NS; ++s) mbar_init(&bars[s], 1);
     for (int s = 0; s < NW; ++s) mbar_init(&wbars[s], Sh::NWARPS);
     fence_barrier_init();
-    for (int s = 0; s < NS && zb + s <= ze; ++s) load_plane(s);
   }
+  // what came before may still run up to here (launch_step); the next launch
+  // may be brought in beside this one
+  grid_wait();
+  grid_release();
+  if (tid == 0)
+    for (int s = 0; s < NS && zb + s <= ze; ++s) load_plane(s);
   __syncthreads();
 
   // a thread whose bounded wait ran out stops waiting and runs the sweep to its

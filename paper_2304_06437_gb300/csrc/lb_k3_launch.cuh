@@ -89,11 +89,10 @@ struct K3Impl {
     const K3Args<R, V> a = args_of(ctx, src);
     const int grid = a.ntx * a.nty * a.ntz;
     const CUtensorMap& tm = ctx->mr.maps[src];
-    if (ctx->g.has_force)
-      k3_step<L, S, R, BX, BY, NS, NPT, true, MINB><<<grid, Sh::NT, Sh::SMEM, ctx->stream>>>(tm, a);
-    else
-      k3_step<L, S, R, BX, BY, NS, NPT, false, MINB><<<grid, Sh::NT, Sh::SMEM, ctx->stream>>>(tm, a);
-    return cudaGetLastError();
+    const bool early = !ctx->mr.shared && grid <= k1_sm_count() * MINB;
+    return launch_step(ctx->g.has_force ? k3_step<L, S, R, BX, BY, NS, NPT, true, MINB>
+                                        : k3_step<L, S, R, BX, BY, NS, NPT, false, MINB>,
+                       grid, Sh::NT, Sh::SMEM, ctx->stream, early, tm, a);
   }
 
   // (no collision: one instantiation serves with and without a force)

@@ -96,6 +96,13 @@ bool moment_plan(lb_ctx* ctx) {
   return true;
 }
 
+MomentRun moment_plan_beside(const lb_ctx* ctx) {
+  MomentRun m = ctx->mr;
+  m.graph = nullptr;
+  m.shared = true;
+  return m;
+}
+
 namespace {
 
 // kMomentGraphSteps steps A -> B -> ... -> A recorded once as a CUDA graph;

@@ -6,8 +6,8 @@
 // for one launch and one memory latency.  What is left bounds the step:
 // instruction issue (large domains) and the launch (small ones).  Per step on
 // one GB300, single-step launches against this form: FP32 cavities of 4096^2 328
-// -> 97 us (173 GLUPS), 1024^2 43.8 -> 8.2, 301 x 257 18.6 -> 2.0, 128 x 96 14.5 ->
-// 1.8; FP64 1024^2 219 -> 173 (bound by the FP64 rate), 301 x 257 72.9 -> 26.0.
+// -> 97 us (173 GLUPS), 1024^2 43.8 -> 8.2, 301 x 257 18.6 -> 1.5, 128 x 96 14.5 ->
+// 1.2; FP64 1024^2 219 -> 173 (bound by the FP64 rate), 301 x 257 72.9 -> 26.0.
 //
 // Between launches the state of a node is its post-collision coefficients, as
 // in lb_k3.cuh (6 values).  The first launch of a run reads populations and the
@@ -85,6 +85,9 @@ __global__ void __launch_bounds__(k4_threads<R>(), 2) k4_steps(const __grid_cons
     return v < 0 ? v + n : v;
   };
 
+  // what came before may still run up to here (launch_step)
+  grid_wait();
+  grid_release();
   {  // read the tile and its ring
     const bool in = tx >= lo_of(0, x0, args.per_x) && tx < hi_of(0, x0, bxa, nx, args.per_x);
     const int rhi = hi_of(0, z0, bza, nz, args.per_z);
@@ -238,7 +241,7 @@ FlatSplit split_run(const Geometry& g, int64_t n, int max_rows, bool fp64) {
 }
 
 template <class R>
-cudaError_t flat_run_as(lb_ctx* ctx, int64_t n) {
+cudaError_t flat_run_as(lb_ctx* ctx, int64_t n, bool beside) {
   const Geometry& g = ctx->g;
   const FlatSplit sp = split_run(g, n, k4_max_rows<R>(), sizeof(R) == 8);
   R* const f = static_cast<R*>(ctx->f);
@@ -265,8 +268,8 @@ cudaError_t flat_run_as(lb_ctx* ctx, int64_t n) {
     a.dst = last ? f : set[i & 1];
     const int grid = a.ntx * div_up(g.nz, a.bz);
     const size_t smem = size_t(a.bz + 2 * a.steps) * 9 * kWidth * sizeof(R);
-    k4_kernel<R>(g.has_force, i == 0 ? 0 : last ? 2 : 1)<<<grid, k4_threads<R>(), smem, ctx->stream>>>(a);
-    e = cudaGetLastError();
+    e = launch_step(k4_kernel<R>(g.has_force, i == 0 ? 0 : last ? 2 : 1), grid, k4_threads<R>(), smem, ctx->stream,
+                    !beside && i > 0 && grid <= 2 * k1_sm_count(), a);
   }
   return e;
 }
@@ -301,8 +304,9 @@ bool flat_plan(lb_ctx* ctx) {
   return true;
 }
 
-cudaError_t flat_run(lb_ctx* ctx, int64_t n) {
-  const cudaError_t e = ctx->storage == LB_F64 ? flat_run_as<double>(ctx, n) : flat_run_as<float>(ctx, n);
+cudaError_t flat_run(lb_ctx* ctx, int64_t n, bool beside) {
+  const cudaError_t e =
+      ctx->storage == LB_F64 ? flat_run_as<double>(ctx, n, beside) : flat_run_as<float>(ctx, n, beside);
   return e == cudaSuccess ? k1_bootstrap(ctx) : e;
 }
 

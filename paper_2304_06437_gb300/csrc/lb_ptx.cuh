@@ -127,4 +127,31 @@ __device__ __forceinline__ void prefetch_tmap(const void* tmap) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(tmap)) : "memory");
 }
 
+// Launches that may begin before the one before them has ended: grid_wait()
+// waits until it has (and its writes are visible), grid_release() lets the next
+// one begin.  Without the launch attribute both do nothing.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// One launch of a chain on a stream.  early: it may begin while the one before
+// it ends, so that its start costs no gap -- for launches of at most one wave,
+// whose blocks find room.  Per step, without -> with: D3Q19 FP32 32^3 4.6 -> 3.9
+// us, 97 x 61 x 113 21.6 -> 20.8, D2Q9 FP32 301 x 257 2.1 -> 1.5, 128 x 96 1.8 ->
+// 1.2.  Not beside other runs: waiting blocks would hold their room.
+template <class... P, class... A>
+cudaError_t launch_step(void (*kernel)(P...), int grid, int threads, size_t smem, cudaStream_t stream, bool early,
+                        const A&... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3(unsigned(grid));
+  c.blockDim = dim3(unsigned(threads));
+  c.dynamicSmemBytes = smem;
+  c.stream = stream;
+  c.attrs = &at;
+  c.numAttrs = early ? 1 : 0;
+  return cudaLaunchKernelEx(&c, kernel, args...);
+}
+
 }  // namespace lbgb
