@@ -39,8 +39,8 @@
 // 16: 104 (136), where three launches over populations and planar fields moved
 // 284 (444).  Measured per step on one GB300, three launches against this form:
 // D2Q9 FP32 4096^2 1126 -> 488 us, 2048 x 1536 with near-contact forces 328 ->
-// 137 us, D3Q19 FP32 192^3 933 -> 766 us (bound by the L1's loads of a pull),
-// 97 x 61 x 113 98.6 -> 76.5 us; FP64 is bound by its arithmetic (1024^2 624 ->
+// 137 us, D3Q19 FP32 192^3 933 -> 427 us (bound by the L1's loads of a pull;
+// 767 with boxes of 8 nodes along x), 97 x 61 x 113 98.6 -> 58.3 us; FP64 is bound by its arithmetic (1024^2 624 ->
 // 613 us).
 //
 // Near-contact interactions (section 2.2), when switched on: the gradient
@@ -404,9 +404,11 @@ int grid_of(int64_t n) {
 }
 
 // The box of a thread block: the power-of-two extents whose boxes cover the
-// domain with the fewest nodes, counting a third of the ring of neighbours that
-// a box reads (most of it from the L2 cache) and rows shorter than 4 nodes as
-// the sectors they half use.
+// domain at the least cost.  The L1's loads bound the pull: a warp's 16-byte
+// load touches one 128-byte line for every 8 nodes of a row and one more for
+// each row (shifted rows straddle lines): 5 lines for rows of 32 nodes, 8 for
+// rows of 8.  The ring of neighbours that a box reads comes from the L2 cache
+// and counts a tenth.
 void plan_boxes(CgGeom& g) {
   double best = 1e300;
   for (int lx = 0; lx <= 8; ++lx)
@@ -415,7 +417,9 @@ void plan_boxes(CgGeom& g) {
       const double bx = 1 << lx, by = 1 << ly, bz = 1 << lz;
       const double tx = std::ceil(g.nx / bx), ty = std::ceil(g.ny / by), tz = std::ceil(g.nz / bz);
       const double ring = (1 + 2 / bx) * (g.ny > 1 ? 1 + 2 / by : 1) * (1 + 2 / bz) - 1;
-      const double cost = tx * ty * tz * (1 + ring / 3) * (lx < 2 ? 2.0 : 1.0);
+      const double row = std::min(bx, 32.0);  // of a warp
+      const double lines = 32 / row * (std::max(1.0, row / 8) + 1);
+      const double cost = tx * ty * tz * (lines / 5 + ring / 10);
       if (cost < best * (1 - 1e-9)) {
         best = cost;
         g.lx = lx;
