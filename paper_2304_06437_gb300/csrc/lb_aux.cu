@@ -9,6 +9,7 @@
 #include <type_traits>
 
 #include "lb_dispatch.cuh"
+#include "lb_widen.cuh"
 
 namespace lbgb {
 namespace {
@@ -35,9 +36,9 @@ inline Layout layout_of(const Geometry& g) {
 }
 
 __device__ __forceinline__ int64_t ioff(const Layout& l, int64_t idx) {
-  const int64_t x = idx % l.nx;
-  const int64_t r = idx / l.nx;
-  return x + r * l.pitch;
+  // 32-bit division where it serves (64-bit is a long instruction sequence)
+  const int64_t r = idx >> 32 ? idx / l.nx : int64_t(uint32_t(idx) / uint32_t(l.nx));
+  return idx + r * (l.pitch - l.nx);
 }
 
 // user vector component k -> internal axis
@@ -60,14 +61,11 @@ __global__ void set_pop_kernel(Layout l, const double* __restrict__ f, S* __rest
 }
 
 template <class L, class S, class R>
-__global__ void get_pop_kernel(Layout l, const S* __restrict__ ft, double* __restrict__ f, double rho0) {
+__global__ void get_pop_kernel(Layout l, const S* ft, double* f, ShellSums sums) {
   for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < l.n;
        idx += (int64_t)gridDim.x * blockDim.x) {
     const int64_t o = ioff(l, idx);
-    static_for<0, L::Q>([&](auto A_) {
-      constexpr int a = decltype(A_)::value;
-      f[a * l.n + idx] = static_cast<double>(load_as<S, R>(ft[a * l.vol + o])) + weight<L>(a) * rho0;
-    });
+    widen_populations<L, S, R>(ft + o, l.vol, f + idx, l.n, sums);
   }
 }
 
@@ -170,7 +168,7 @@ struct Sum2 {
     lo += (hi - (s - bp)) + (x - bp);
     hi = s;
   }
-  __device__ __forceinline__ double value() const { return double(hi) + double(lo); }
+  __device__ __forceinline__ double value() const { return widen(hi) + widen(lo); }
 };
 
 template <class L, class S, class R>
@@ -206,9 +204,12 @@ __device__ __forceinline__ void node_sums(const S* __restrict__ ft, int64_t vol,
   }
 }
 
-template <class L, class S, class R>
+// UNIT: rho0 = 1, where the division by it is left out at compile time (x / 1 is
+// x; as a branch the compiler computes the FP64 division ahead of it, which
+// took most of these kernels' time)
+template <class L, class S, class R, bool UNIT>
 // nodes [n0, n1) into element idx - n0 of each output component (cs apart)
-__global__ void moments_kernel(Layout l, const S* __restrict__ ft, double rho0, double Fx, double Fy, double Fz,
+__global__ void moments_kernel(Layout l, const S* __restrict__ ft, double rho0, double hFx, double hFy, double hFz,
                                double* __restrict__ rho, double* __restrict__ u, int64_t n0, int64_t n1,
                                int64_t cs) {
   for (int64_t idx = n0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < n1;
@@ -219,12 +220,11 @@ __global__ void moments_kernel(Layout l, const S* __restrict__ ft, double rho0, 
     node_sums<L, S, R>(ft, l.vol, o, dr, j, bad);
     if (rho) rho[idx - n0] = rho0 + dr;
     if (u) {
-      const double Fi[3] = {Fx, Fy, Fz};
+      const double hF[3] = {hFx, hFy, hFz};
       for (int k = 0; k < L::D; ++k) {
         const int ax = user_axis<L>(k);
-        // x / 1 is x exactly: the common rho0 = 1 skips the FP64 division
-        const double v = j[ax] + 0.5 * Fi[ax];
-        u[k * cs + (idx - n0)] = rho0 == 1.0 ? v : v / rho0;
+        const double v = j[ax] + hF[ax];
+        u[k * cs + (idx - n0)] = UNIT ? v : v / rho0;
       }
     }
   }
@@ -251,13 +251,14 @@ __global__ void region_kernel(Layout l, int ny, const S* __restrict__ ft, double
 // non-finite count]; u in internal axes.  Fixed grid + tree order.
 constexpr int kRedFields = 7;
 
-template <class L, class S, class R>
+template <class L, class S, class R, bool UNIT>
 __global__ void __launch_bounds__(kThreads) reduce_kernel(Layout l, const S* __restrict__ ft, double rho0,
-                                                          double Fx, double Fy, double Fz,
+                                                          double hFx, double hFy, double hFz,
                                                           float* __restrict__ uprev, int residual,
                                                           double* __restrict__ partial) {
   double acc[kRedFields] = {0, 0, 0, 0, 0, 0, 0};
-  const double Fi[3] = {Fx, Fy, Fz};
+  const double hF[3] = {hFx, hFy, hFz};
+  int64_t nbad = 0;
   for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < l.n;
        idx += (int64_t)gridDim.x * blockDim.x) {
     const int64_t o = ioff(l, idx);
@@ -268,18 +269,19 @@ __global__ void __launch_bounds__(kThreads) reduce_kernel(Layout l, const S* __r
     acc[1] += j[0];
     acc[2] += j[1];
     acc[3] += j[2];
-    acc[6] += bad ? 1.0 : 0.0;
+    nbad += bad;
     if (residual) {
       for (int k = 0; k < 3; ++k) {
-        const double vk = j[k] + 0.5 * Fi[k];
-        const double uk = rho0 == 1.0 ? vk : vk / rho0;  // x / 1 is x exactly
-        const double prev = static_cast<double>(uprev[k * l.n + idx]);
-        acc[4] += (uk - prev) * (uk - prev);
-        acc[5] += uk * uk;
+        const double vk = j[k] + hF[k];
+        const double uk = UNIT ? vk : vk / rho0;
+        const double du = uk - widen(uprev[k * l.n + idx]);
+        acc[4] = fma(du, du, acc[4]);
+        acc[5] = fma(uk, uk, acc[5]);
         uprev[k * l.n + idx] = static_cast<float>(uk);
       }
     }
   }
+  acc[6] = static_cast<double>(nbad);
   __shared__ double sh[kRedFields][kThreads];
   for (int k = 0; k < kRedFields; ++k) sh[k][threadIdx.x] = acc[k];
   __syncthreads();
@@ -340,7 +342,7 @@ cudaError_t aux_get_populations(lb_ctx* ctx, double* f_dev) {
       using S = typename decltype(St)::type;
       using R = typename decltype(Rt)::type;
       get_pop_kernel<L, S, R><<<grid_for(l.n), kThreads, 0, ctx->stream>>>(
-          l, static_cast<const S*>(ctx->f), f_dev, ctx->g.rho0);
+          l, static_cast<const S*>(ctx->f), f_dev, shell_sums<L>(ctx->g.rho0));
     });
   });
   return cudaGetLastError();
@@ -394,8 +396,9 @@ cudaError_t aux_moments_range(lb_ctx* ctx, double* rho, double* u, int64_t n0, i
     dispatch_storage(ctx->storage, [&](auto St, auto Rt) {
       using S = typename decltype(St)::type;
       using R = typename decltype(Rt)::type;
-      moments_kernel<L, S, R><<<grid_for(n1 - n0), kThreads, 0, ctx->stream>>>(
-          l, static_cast<const S*>(ctx->f), ctx->g.rho0, F[0], F[1], F[2], rho, u, n0, n1, cs);
+      const auto kernel = ctx->g.rho0 == 1.0 ? moments_kernel<L, S, R, true> : moments_kernel<L, S, R, false>;
+      kernel<<<grid_for(n1 - n0), kThreads, 0, ctx->stream>>>(l, static_cast<const S*>(ctx->f), ctx->g.rho0,
+                                                              0.5 * F[0], 0.5 * F[1], 0.5 * F[2], rho, u, n0, n1, cs);
     });
   });
   return cudaGetLastError();
@@ -440,8 +443,9 @@ cudaError_t aux_reduce_enqueue(lb_ctx* ctx, cudaStream_t stream, double* dev_out
     dispatch_storage(ctx->storage, [&](auto St, auto Rt) {
       using S = typename decltype(St)::type;
       using R = typename decltype(Rt)::type;
-      reduce_kernel<L, S, R><<<kRedBlocks, kThreads, 0, stream>>>(
-          l, static_cast<const S*>(ctx->f), ctx->g.rho0, F[0], F[1], F[2], ctx->d_uprev, residual ? 1 : 0,
+      const auto kernel = ctx->g.rho0 == 1.0 ? reduce_kernel<L, S, R, true> : reduce_kernel<L, S, R, false>;
+      kernel<<<kRedBlocks, kThreads, 0, stream>>>(
+          l, static_cast<const S*>(ctx->f), ctx->g.rho0, 0.5 * F[0], 0.5 * F[1], 0.5 * F[2], ctx->d_uprev, residual ? 1 : 0,
           ctx->d_red);
     });
   });

@@ -62,6 +62,7 @@
 #include <new>
 
 #include "lb_dispatch.cuh"
+#include "lb_widen.cuh"
 
 namespace lbgb {
 namespace {
@@ -354,12 +355,9 @@ __global__ void cg_init_kernel(CgGeom g, const double* __restrict__ rr, const do
 }
 
 template <class L, class S, class R>
-__global__ void cg_get_kernel(CgGeom g, const S* __restrict__ fs, double rho0, double* __restrict__ f) {
+__global__ void cg_get_kernel(CgGeom g, const S* fs, ShellSums sums, double* f) {
   for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < g.n; i += int64_t(gridDim.x) * blockDim.x)
-    static_for<0, L::Q>([&](auto A_) {
-      constexpr int a = decltype(A_)::value;
-      f[a * g.n + i] = double(load_as<S, R>(fs[a * g.n + i])) + 0.5 * weight<L>(a) * rho0;
-    });
+    widen_populations<L, S, R>(fs + i, g.n, f + i, g.n, sums);
 }
 
 template <class L, class S, class R>
@@ -376,23 +374,40 @@ __global__ void cg_fields_kernel(CgGeom g, const S* __restrict__ fr, const S* __
                                  int d, double* __restrict__ rr, double* __restrict__ rb, double* __restrict__ u) {
   for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < g.n; i += int64_t(gridDim.x) * blockDim.x) {
     double sr = 0.0, sb = 0.0, j[3] = {0, 0, 0};
+    // (the terms with a zero component leave a finite sum as it is; they are
+    // added only where a population is not finite)
+    bool finite = true;
     static_for<0, L::Q>([&](auto A_) {
       constexpr int a = decltype(A_)::value;
-      const double r = double(load_as<S, R>(fr[a * g.n + i])), b = double(load_as<S, R>(fb[a * g.n + i]));
+      constexpr int cx = L::cx(a), cy = L::cy(a), cz = L::cz(a);
+      const double r = widen(load_as<S, R>(fr[a * g.n + i])), b = widen(load_as<S, R>(fb[a * g.n + i]));
+      finite = finite && isfinite(r) && isfinite(b);
       sr += r;
       sb += b;
-      j[0] += L::cx(a) * (r + b);
-      j[1] += L::cy(a) * (r + b);
-      j[2] += L::cz(a) * (r + b);
+      const double t = r + b;
+      if constexpr (cx != 0) j[0] += cx > 0 ? t : -t;
+      if constexpr (cy != 0) j[1] += cy > 0 ? t : -t;
+      if constexpr (cz != 0) j[2] += cz > 0 ? t : -t;
     });
+    if (!finite) {
+      j[0] = j[1] = j[2] = 0.0;
+      static_for<0, L::Q>([&](auto A_) {
+        constexpr int a = decltype(A_)::value;
+        const double t = double(load_as<S, R>(fr[a * g.n + i])) + double(load_as<S, R>(fb[a * g.n + i]));
+        j[0] += L::cx(a) * t;
+        j[1] += L::cy(a) * t;
+        j[2] += L::cz(a) * t;
+      });
+    }
     if (rr) rr[i] = sr + 0.5 * rho0;
     if (rb) rb[i] = sb + 0.5 * rho0;
     if (u) {
-      u[i] = j[0] / rho0;
-      if (d == 2) u[g.n + i] = j[2] / rho0;
+      // (rho0 = 1: lb_cg_create)
+      u[i] = j[0];
+      if (d == 2) u[g.n + i] = j[2];
       else {
-        u[g.n + i] = j[1] / rho0;
-        u[2 * g.n + i] = j[2] / rho0;
+        u[g.n + i] = j[1];
+        u[2 * g.n + i] = j[2];
       }
     }
   }
@@ -626,7 +641,7 @@ int lb_cg_get_populations(lb_cg* c, double* fr, double* fb, int32_t on_device) {
       using S = typename decltype(St)::type;
       using R = typename decltype(Rt)::type;
       cg_get_kernel<L, S, R><<<grid_of(c->g.n), kCgThreads, 0, c->stream>>>(
-          c->g, static_cast<const S*>(k == 0 ? c->fr : c->fb), c->rho0, d);
+          c->g, static_cast<const S*>(k == 0 ? c->fr : c->fb), shell_sums<L>(0.5 * c->rho0), d);
     });
     rc = rc_of(cudaGetLastError());
     if (!on_device) {
