@@ -1082,11 +1082,17 @@ __global__ void __launch_bounds__(K1Shape<L, S, R, BX, BY, NS, WB, NXW, TS, MINB
 template <class L, class S, class R, int BX, int BY, bool FORCE, bool INC = false>
 __global__ void __launch_bounds__(256) k1_bootstrap(const __grid_constant__ K1Args<R> args) {
   constexpr int Q = L::Q;
-  const int64_t n = int64_t(args.nx) * args.ny * args.nz;
-  for (int64_t idx = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; idx < n; idx += int64_t(gridDim.x) * blockDim.x) {
-    const int x = int(idx % args.nx);
-    const int y = int((idx / args.nx) % args.ny);
-    const int z = int(idx / (int64_t(args.nx) * args.ny));
+  // a warp takes a row's columns of a few bricks at a time: all of them where
+  // the row is an edge of its bricks, else the two edge columns of each brick
+  // (D3Q19 in 32 x 16 bricks: one node in six is at an edge).  Against a pass over
+  // all nodes, each with three 64-bit divisions, a run's share of the shell and
+  // its end: 256^3 D3Q19 FP32 684 -> 642 us, D3Q27 1426 -> 1337, FP16 160^3 247 ->
+  // 224, D2Q9 4096^2 417 -> 340
+  constexpr int CB = BX >= 256 ? 1 : 256 / BX, CH = CB * BX;
+  const int chunks = (args.nx + CH - 1) / CH;
+  const int64_t items = int64_t(chunks) * args.ny * args.nz;
+  const int lane = threadIdx.x % 32;
+  auto node = [&](const int x, const int y, const int z) {
     const int bI = x / BX, bJ = y / BY, bK = z / args.bz;
     const int x0 = bI * BX, y0 = bJ * BY, z0 = bK * args.bz;
     const int bxa = min(BX, args.nx - x0), bya = min(BY, args.ny - y0), z1 = min(z0 + args.bz, args.nz);
@@ -1096,7 +1102,7 @@ __global__ void __launch_bounds__(256) k1_bootstrap(const __grid_constant__ K1Ar
     const bool eN = y == y0 + bya - 1 && (y0 + bya < args.ny || args.per[1]);
     const bool eD = z == z0 && (z0 > 0 || args.per[2] || args.zlink[0]);
     const bool eU = z == z1 - 1 && (z1 < args.nz || args.per[2] || args.zlink[1]);
-    if (!(eW || eE || eS || eN || eD || eU)) continue;
+    if (!(eW || eE || eS || eN || eD || eU)) return;
     const int64_t o = x + args.pitch * (y + int64_t(args.ny) * z);
     const unsigned faces = (eW ? kFaceW : 0u) | (eE ? kFaceE : 0u) | (eS ? kFaceS : 0u) | (eN ? kFaceN : 0u) |
                            (eD ? kFaceD : 0u) | (eU ? kFaceU : 0u);
@@ -1113,6 +1119,22 @@ __global__ void __launch_bounds__(256) k1_bootstrap(const __grid_constant__ K1Ar
         fr[a] = load_as<S, R>(fg[a * args.vol + o]);
       });
       export_node<L, S, R, FORCE, true>(args, fr, x, y, z, faces, bI, bJ, bK);
+    }
+  };
+  for (int64_t it = (blockIdx.x * int64_t(blockDim.x) + threadIdx.x) / 32; it < items;
+       it += int64_t(gridDim.x) * (blockDim.x / 32)) {
+    const uint32_t row = uint32_t(it / chunks);
+    const int c0 = int(it - int64_t(row) * chunks) * CH, c1 = min(c0 + CH, args.nx);
+    const int z = int(row / uint32_t(args.ny)), y = int(row - uint32_t(z) * uint32_t(args.ny));
+    const int ty = y % BY, tz = z % args.bz;
+    if (ty == 0 || ty == BY - 1 || y == args.ny - 1 || tz == 0 || tz == args.bz - 1 || z == args.nz - 1) {
+      for (int x = c0 + lane; x < c1; x += 32) node(x, y, z);
+    } else {
+      for (int k = lane; k < 2 * CB; k += 32) {
+        const int x0 = c0 + k / 2 * BX, x1 = min(x0 + BX, args.nx) - 1;
+        // a brick of one column has one edge
+        if (x0 < args.nx && (k % 2 == 0 || x1 > x0)) node(k % 2 ? x1 : x0, y, z);
+      }
     }
   }
 }

@@ -40,6 +40,15 @@ struct K1Variant {
 const K1Variant* k1_ctx_variant(lb_ctx* ctx);
 int k1_sm_count();
 
+// blocks of eight warps for k1_bootstrap's items: rows in pieces of about 256
+// columns, one to a warp
+inline int k1_bootstrap_blocks(const Geometry& g, int bx) {
+  const int ch = bx >= 256 ? bx : 256 / bx * bx;
+  const int64_t items = int64_t((g.nx + ch - 1) / ch) * g.ny * g.nz;
+  const int64_t blocks = (items + 7) / 8;
+  return int(blocks < 152 * 32 ? blocks : 152 * 32);
+}
+
 template <class R>
 K1Args<R> k1_make_args(lb_ctx* ctx, int cur_parity, int next_parity) {
   const Geometry& g = ctx->g;
@@ -120,13 +129,11 @@ struct K1Impl {
   static cudaError_t bootstrap(lb_ctx* ctx) {
     // fill the parity the next step reads
     K1Args<R> a = k1_make_args<R>(ctx, 1 - ctx->parity, ctx->parity);
-    const int64_t n = int64_t(ctx->g.nx) * ctx->g.ny * ctx->g.nz;
-    int64_t blocks = (n + 255) / 256;
-    if (blocks > 152 * 32) blocks = 152 * 32;
+    const int blocks = k1_bootstrap_blocks(ctx->g, BX);
     if (ctx->g.has_force)
-      k1_bootstrap<L, S, R, BX, BY, true><<<int(blocks), 256, 0, ctx->stream>>>(a);
+      k1_bootstrap<L, S, R, BX, BY, true><<<blocks, 256, 0, ctx->stream>>>(a);
     else
-      k1_bootstrap<L, S, R, BX, BY, false><<<int(blocks), 256, 0, ctx->stream>>>(a);
+      k1_bootstrap<L, S, R, BX, BY, false><<<blocks, 256, 0, ctx->stream>>>(a);
     return cudaGetLastError();
   }
 

@@ -139,10 +139,8 @@ struct LeaveImpl {
 
   static cudaError_t shell(lb_ctx* ctx) {
     K1Args<R> a = k1_make_args<R>(ctx, 1 - ctx->parity, ctx->parity);
-    const int64_t n = int64_t(ctx->g.nx) * ctx->g.ny * ctx->g.nz;
-    const int64_t blocks = std::min<int64_t>((n + 255) / 256, 152 * 32);
     // the coefficients already hold the forcing: one instantiation serves both
-    k1_bootstrap<L, S, R, BX, BY, false, true><<<int(blocks), 256, 0, ctx->stream>>>(a);
+    k1_bootstrap<L, S, R, BX, BY, false, true><<<k1_bootstrap_blocks(ctx->g, BX), 256, 0, ctx->stream>>>(a);
     return cudaGetLastError();
   }
 
