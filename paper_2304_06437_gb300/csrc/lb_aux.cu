@@ -36,9 +36,9 @@ inline Layout layout_of(const Geometry& g) {
 }
 
 __device__ __forceinline__ int64_t ioff(const Layout& l, int64_t idx) {
-  // 32-bit division where it serves (64-bit is a long instruction sequence)
-  const int64_t r = idx >> 32 ? idx / l.nx : int64_t(uint32_t(idx) / uint32_t(l.nx));
-  return idx + r * (l.pitch - l.nx);
+  const int64_t x = idx % l.nx;
+  const int64_t r = idx / l.nx;
+  return x + r * l.pitch;
 }
 
 // user vector component k -> internal axis
@@ -61,7 +61,7 @@ __global__ void set_pop_kernel(Layout l, const double* __restrict__ f, S* __rest
 }
 
 template <class L, class S, class R>
-__global__ void get_pop_kernel(Layout l, const S* ft, double* f, ShellSums sums) {
+__global__ void get_pop_kernel(Layout l, const S* ft, double* f, const __grid_constant__ ShellSums sums) {
   for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < l.n;
        idx += (int64_t)gridDim.x * blockDim.x) {
     const int64_t o = ioff(l, idx);
@@ -252,7 +252,7 @@ __global__ void region_kernel(Layout l, int ny, const S* __restrict__ ft, double
 constexpr int kRedFields = 7;
 
 template <class L, class S, class R, bool UNIT>
-__global__ void __launch_bounds__(kThreads) reduce_kernel(Layout l, const S* __restrict__ ft, double rho0,
+__global__ void __launch_bounds__(kThreads, 4) reduce_kernel(Layout l, const S* __restrict__ ft, double rho0,
                                                           double hFx, double hFy, double hFz,
                                                           float* __restrict__ uprev, int residual,
                                                           double* __restrict__ partial) {
