@@ -44,8 +44,7 @@ struct lb_batch {
   };
   std::vector<Class> classes;
   std::vector<int> runs;    // members that calls of several steps run on their own,
-  std::vector<int> lane;    // the stream (of lanes) that each of them runs on,
-  std::vector<lbgb::MomentRun> beside;  // its plan there (3D), and
+  std::vector<int> lane;    // the stream (of lanes) that each of them runs on, and
   std::vector<Class> rest;  // the classes of the others
   int* d_status = nullptr;
   cudaGraphExec_t graph = nullptr;       // two steps of all classes, and
@@ -431,7 +430,6 @@ int lb_batch_create(lb_ctx* const* ctxs, int32_t n, void* stream, lb_batch** out
       const size_t k = std::min_element(load.begin(), load.end()) - load.begin();
       b->lane.push_back(int(k));
       load[k] += ctxs[i]->n_nodes;
-      b->beside.push_back(ctxs[i]->g.d == 3 ? moment_plan_beside(ctxs[i]) : MomentRun{});
     }
     for (size_t k = 0; k < lanes && rc == LB_OK; ++k) {
       cudaStream_t st = nullptr;
@@ -481,16 +479,10 @@ int lb_batch_step(lb_batch* b, int64_t n) {
     for (cudaStream_t st : b->lanes) LB_BTRY(cudaStreamWaitEvent(st, b->done, 0));
     for (size_t k = 0; k < b->runs.size() && rc == LB_OK; ++k) {
       lb_ctx* x = b->ctxs[b->runs[k]];
-      // the launches of a run go to the stream of the context, by its plan
+      // the launches of a run go to the stream of the context
       const cudaStream_t own = x->stream;
       x->stream = b->lanes[b->lane[k]];
-      if (x->g.d == 3) {
-        std::swap(x->mr, b->beside[k]);
-        rc = cuda_rc(moment_run(x, n));
-        std::swap(x->mr, b->beside[k]);
-      } else {
-        rc = cuda_rc(flat_run(x, n, true));
-      }
+      rc = cuda_rc(x->g.d == 3 ? moment_run_beside(x, n) : flat_run(x, n, true));
       x->stream = own;
       x->steps_done += n;
     }
@@ -582,8 +574,6 @@ void lb_batch_destroy(lb_batch* b) {
   if (b->stream) cudaStreamSynchronize(b->stream);
   if (b->graph) cudaGraphExecDestroy(b->graph);
   if (b->rest_graph) cudaGraphExecDestroy(b->rest_graph);
-  for (auto& m : b->beside)
-    if (m.graph) cudaGraphExecDestroy(m.graph);
   for (auto& c : b->classes) free_class(c);
   for (auto& c : b->rest) free_class(c);
   if (b->d_status) cudaFree(b->d_status);

@@ -101,6 +101,7 @@ struct lb_ctx {
   cudaGraphExec_t step_graph = nullptr;
   int graph_parity = 0;
   lbgb::MomentRun mr;
+  lbgb::MomentRun beside; // the same beside other runs (a batch's), once needed
   int flat_state = 0;     // runs of 2D domains: 0 not planned yet, 1 usable, -1 not
 };
 
@@ -158,9 +159,9 @@ bool moment_plan(lb_ctx* ctx);
 // n >= 2 steps of a planned context
 cudaError_t moment_run(lb_ctx* ctx, int64_t n);
 void drop_moment_run(lb_ctx* ctx);
-// the run of a planned context beside others: recorded steps of its own, whose
-// launches keep no room for the next, for the context while it runs so
-MomentRun moment_plan_beside(const lb_ctx* ctx);
+// the same while other runs share the device: recorded steps of its own, whose
+// launches keep no room for the next
+cudaError_t moment_run_beside(lb_ctx* ctx, int64_t n);
 // TMA descriptor of nf fields of the arithmetic type at base, boxes of bx x by
 // x 1 x nf (lb_capi.cu)
 bool make_field_map(lb_ctx* ctx, CUtensorMap* map, void* base, int nf, int bx, int by);

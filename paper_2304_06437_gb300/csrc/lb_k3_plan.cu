@@ -96,13 +96,6 @@ bool moment_plan(lb_ctx* ctx) {
   return true;
 }
 
-MomentRun moment_plan_beside(const lb_ctx* ctx) {
-  MomentRun m = ctx->mr;
-  m.graph = nullptr;
-  m.shared = true;
-  return m;
-}
-
 namespace {
 
 // kMomentGraphSteps steps A -> B -> ... -> A recorded once as a CUDA graph;
@@ -164,9 +157,24 @@ cudaError_t moment_run(lb_ctx* ctx, int64_t n) {
   return e;
 }
 
+cudaError_t moment_run_beside(lb_ctx* ctx, int64_t n) {
+  if (!moment_plan(ctx)) return cudaErrorInvalidValue;
+  if (ctx->beside.state != 1) {
+    ctx->beside = ctx->mr;
+    ctx->beside.graph = nullptr;
+    ctx->beside.shared = true;
+  }
+  std::swap(ctx->mr, ctx->beside);
+  const cudaError_t e = moment_run(ctx, n);
+  std::swap(ctx->mr, ctx->beside);
+  return e;
+}
+
 void drop_moment_run(lb_ctx* ctx) {
-  if (ctx->mr.graph) cudaGraphExecDestroy(ctx->mr.graph);
-  ctx->mr = MomentRun{};
+  for (MomentRun* m : {&ctx->mr, &ctx->beside}) {
+    if (m->graph) cudaGraphExecDestroy(m->graph);
+    *m = MomentRun{};
+  }
 }
 
 }  // namespace lbgb
