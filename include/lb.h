@@ -318,9 +318,9 @@ LB_API int lb_autotune(lb_ctx* ctx, int32_t steps, lb_tune_entry* table, int32_t
  * sweeps of up to 256 planes; where a class would then have fewer than two
  * bricks per persistent CTA, its members' sweeps are halved (down to 64
  * planes) until it has.  Classes run on parallel branches of the graph.
- * Calls of four or more steps take members of at least 65536 nodes (2D: 16384)
- * through the runs that lb_step() has for several steps, on streams of the
- * batch and beside the classes of the other members.
+ * Calls of four or more steps take the largest members, as many as have 160 Ki
+ * nodes (2D: 64 Ki) on average, through the runs that lb_step() has for several steps, on
+ * streams of the batch and beside the classes of the other members.
  * stream: cudaStream_t for the batch's work, NULL = a library-owned stream.
  * Errors: LB_E_INVAL (NULL, duplicates, mixed devices), LB_E_UNSUPPORTED,
  * LB_E_NOMEM, LB_E_CUDA. */

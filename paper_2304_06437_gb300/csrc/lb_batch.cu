@@ -255,14 +255,27 @@ int split_for_balance(lb_batch& b, lb_batch::Class& c) {
   return LB_OK;
 }
 
-// Whether calls of several steps run a member on its own.  A step of such a run
-// costs the host about a microsecond (a recorded graph of eight launches in
-// 3D, a launch for up to eight steps in 2D), which a member has to be worth on
-// the device; the classes carry the smaller ones at no cost of their own.
-bool runs_alone(lb_ctx* x) {
-  constexpr int64_t kMin3d = 65536, kMin2d = 16384;
-  if (x->n_nodes < (x->g.d == 2 ? kMin2d : kMin3d)) return false;
-  return moment_plan(x) || flat_plan(x);
+// The members that calls of several steps run on their own, the largest first:
+// as many as keep kMeanRunNodes on average, a 2D node counting for 2.5 (its runs
+// take several steps per launch).  A step of such a run costs the host about a
+// microsecond and the device a launch of few bricks, which the members together
+// have to be worth; the classes carry many small ones at less.  100 steps, classes
+// against runs: 24 D3Q19 members of 48^3 11.7 / 12.6 ms, 48 D2Q9 members of 300^2
+// 12.3 / 3.6, 24 mixed members of 17^3 to 115^3 and 36^2 to 958^2 41 / 17.
+std::vector<int> runs_alone(const std::vector<lb_ctx*>& ctxs) {
+  constexpr double kMeanRunNodes = 160 * 1024;
+  std::vector<int> order(ctxs.size()), runs;
+  for (size_t i = 0; i < order.size(); ++i) order[i] = int(i);
+  auto weight = [&](int i) { return double(ctxs[i]->n_nodes) * (ctxs[i]->g.d == 2 ? 2.5 : 1.0); };
+  std::stable_sort(order.begin(), order.end(), [&](int i, int j) { return weight(i) > weight(j); });
+  double sum = 0.0;
+  for (int i : order) {
+    if (sum + weight(i) < kMeanRunNodes * double(runs.size() + 1)) break;
+    if (!moment_plan(ctxs[i]) && !flat_plan(ctxs[i])) continue;
+    sum += weight(i);
+    runs.push_back(i);
+  }
+  return runs;
 }
 
 // One step (k = 0 or 1 of the captured pair) of every class.  Classes are
@@ -417,13 +430,10 @@ int lb_batch_create(lb_ctx* const* ctxs, int32_t n, void* stream, lb_batch** out
       if (cudaEventCreateWithFlags(&b->ctx_ev[i], cudaEventDisableTiming) != cudaSuccess) rc = LB_E_CUDA;
     if (rc != LB_OK) break;
     if ((rc = capture_pair(*b, b->classes, &b->graph)) != LB_OK) break;
-    // members that run alone, the largest first, and the classes without them
-    for (int i = 0; i < n; ++i)
-      if (runs_alone(ctxs[i])) b->runs.push_back(i);
+    // members that run alone, and the classes without them
+    b->runs = runs_alone(b->ctxs);
     // (eight lanes: the streams that the device runs side by side by default),
     // each to the least loaded
-    std::stable_sort(b->runs.begin(), b->runs.end(),
-                     [&](int i, int j) { return ctxs[i]->n_nodes > ctxs[j]->n_nodes; });
     const size_t lanes = std::min<size_t>(b->runs.size(), 8);
     std::vector<int64_t> load(lanes, 0);
     for (int i : b->runs) {

@@ -54,3 +54,37 @@ def test_members_as_if_alone(small_only, large_only):
             assert s.info()["steps_done"] == 28 + (i % 2)
     for s in members:
         s.close()
+
+
+def test_small_members_beside_a_large_one_as_if_alone():
+    """One large member keeps the mean size up: 2D, 16-bit and one-column members
+    of every storage run on their own too; forms without a run stay in classes."""
+    import paper_2304_06437_gb300 as lb
+    from paper_2304_06437_gb300 import build
+    build.build()
+    specs = SPECS + [("D3Q19", (110, 101, 97), "f32", "lid"), ("D2Q9", (31, 1, 1), "f32", "periodic"),
+                     ("D2Q9", (77, 31, 1), "bf16s", "lid"), ("D3Q27", (9, 8, 7), "bf16s", "walls")]
+
+    def make(i):
+        lat, dims, storage, fname = specs[i]
+        faces, wall_u = faces_for(lat, fname)
+        s = lb.Solver(lat, dims, 0.58 + 0.02 * i, faces=faces, wall_u=wall_u, storage=storage,
+                      force=(2e-5, 1e-5, 0.0) if fname == "duct" else (0, 0, 0))
+        s.set_populations(np.ascontiguousarray(random_state(lat, dims, 40 + i)))
+        return s
+
+    want = []
+    for i in range(len(specs)):
+        with make(i) as s:
+            for _ in range(17):
+                s.step(1)
+            want.append(s.get_populations())
+    members = [make(i) for i in range(len(specs))]
+    with lb.Batch(members) as b:
+        for n in (6, 1, 10):
+            b.step(n)
+        b.sync()
+        for s, f, spec in zip(members, want, specs):
+            assert np.array_equal(s.get_populations(), f), spec
+    for s in members:
+        s.close()
