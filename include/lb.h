@@ -238,6 +238,19 @@ typedef struct {
 LB_API int lb_plan_fused(int32_t lattice, int32_t storage, const int64_t dims[3], const int32_t tile[3],
                          int32_t sms, lb_plan_t* out);
 
+/* How lb_step(n) divides a run of a 2D domain in FP64 or FP32 storage into
+ * launches of several steps each (no device is touched): an even number of
+ * launches, the first of them steps_first steps long and the last steps_last,
+ * on tiles of tile_rows rows that are read with a ring of as many rows as the
+ * launch has steps (max_rows: what shared memory holds).  n >= 2; sms as for
+ * lb_plan_fused().  Errors: LB_E_INVAL, LB_E_UNSUPPORTED. */
+typedef struct {
+  int64_t launches;
+  int32_t steps_first, steps_last;
+  int32_t tile_rows, max_rows;
+} lb_flat_plan_t;
+LB_API int lb_plan_flat(int32_t storage, const int64_t dims[3], int64_t n, int32_t sms, lb_flat_plan_t* out);
+
 /* Allocation-free step for callers that cannot let a library call
  * cudaMalloc (device memory owned by another allocator or a fixed budget, or
  * loops that must not enter the driver's allocator).  The paper has no

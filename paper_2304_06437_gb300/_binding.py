@@ -101,6 +101,11 @@ class lb_plan_t(ctypes.Structure):
                 ("shell_elems_per_parity", ctypes.c_int64)]
 
 
+class lb_flat_plan_t(ctypes.Structure):
+    _fields_ = [("launches", ctypes.c_int64), ("steps_first", ctypes.c_int32), ("steps_last", ctypes.c_int32),
+                ("tile_rows", ctypes.c_int32), ("max_rows", ctypes.c_int32)]
+
+
 class lb_batch_info_t(ctypes.Structure):
     _fields_ = [
         ("n_domains", ctypes.c_int32),
@@ -162,6 +167,7 @@ SIGNATURES = {
     "lb_cg_set_nci": (ctypes.c_int, [_vp, ctypes.c_double, ctypes.c_double, ctypes.c_int32]),
     "lb_plan_fused": (ctypes.c_int, [ctypes.c_int32, ctypes.c_int32, _i64p, _P(ctypes.c_int32), ctypes.c_int32,
                                      _P(lb_plan_t)]),
+    "lb_plan_flat": (ctypes.c_int, [ctypes.c_int32, _i64p, ctypes.c_int64, ctypes.c_int32, _P(lb_flat_plan_t)]),
     "lb_halo_bytes": (ctypes.c_int, [_vp, _i64p]),
     "lb_halo_pack": (ctypes.c_int, [_vp, ctypes.c_int32, _vp]),
     "lb_halo_unpack": (ctypes.c_int, [_vp, ctypes.c_int32, _vp]),

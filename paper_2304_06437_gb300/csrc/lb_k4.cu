@@ -216,17 +216,20 @@ struct FlatSplit {
   int64_t launches = 0;
   int bz = 0;
 };
-FlatSplit split_run(const Geometry& g, int64_t n, int max_rows, bool fp64) {
+FlatSplit split_run(int64_t nx, int64_t nz, int64_t n, int max_rows, bool fp64, int sm_count) {
   FlatSplit best;
   double best_cost = 1e300;
   const double read = fp64 ? 0.65 : 0.12, step = fp64 ? 2.3 : 0.053;
-  const double sms = k1_sm_count();
+  const double sms = sm_count;
   for (int T = 1; T <= kMaxSteps; ++T) {
     const int64_t launches = 2 * ((n + 2 * T - 1) / (2 * T));
+    // an odd n in single steps leaves none for the last launch, which has to
+    // write the populations
+    if (launches > n) continue;
     const int steps = int((n + launches - 1) / launches);
-    const int64_t ntx = div_up(g.nx, kWidth - 2 * steps);
+    const int64_t ntx = (nx + kWidth - 2 * steps - 1) / (kWidth - 2 * steps);
     for (int bz = 8; bz + 2 * steps <= max_rows; bz += 8) {
-      const double tiles = double(ntx) * div_up(g.nz, bz);
+      const double tiles = double(ntx) * double((nz + bz - 1) / bz);
       const double tile = 1.0 + read * (bz + 2 * steps) + step * steps * (bz + steps - 1);
       const double rounds = tiles <= sms ? 0.9 : std::max(1.7, tiles / (2 * sms) + 0.5);
       const double cost = double(launches) * (3.0 + rounds * tile);
@@ -240,10 +243,14 @@ FlatSplit split_run(const Geometry& g, int64_t n, int max_rows, bool fp64) {
   return best;
 }
 
+// steps of launch i: as even as they come, the longer launches first
+int launch_steps(int64_t n, int64_t launches, int64_t i) { return int(n / launches + (i < n % launches ? 1 : 0)); }
+
 template <class R>
 cudaError_t flat_run_as(lb_ctx* ctx, int64_t n, bool beside) {
   const Geometry& g = ctx->g;
-  const FlatSplit sp = split_run(g, n, k4_max_rows<R>(), sizeof(R) == 8);
+  const FlatSplit sp = split_run(g.nx, g.nz, n, k4_max_rows<R>(), sizeof(R) == 8, k1_sm_count());
+  if (sp.launches < 2) return cudaErrorInvalidValue;
   R* const f = static_cast<R*>(ctx->f);
   R* const set[2] = {f + set_a_at(g), f};
   K4Args<R> a;
@@ -261,7 +268,7 @@ cudaError_t flat_run_as(lb_ctx* ctx, int64_t n, bool beside) {
   cudaError_t e = cudaSuccess;
   for (int64_t i = 0; i < sp.launches && e == cudaSuccess; ++i) {
     const bool last = i == sp.launches - 1;
-    a.steps = int(n / sp.launches + (i < n % sp.launches ? 1 : 0));
+    a.steps = launch_steps(n, sp.launches, i);
     a.bx = kWidth - 2 * a.steps;
     a.ntx = div_up(g.nx, a.bx);
     a.src = i == 0 ? f : set[(i - 1) & 1];
@@ -311,3 +318,20 @@ cudaError_t flat_run(lb_ctx* ctx, int64_t n, bool beside) {
 }
 
 }  // namespace lbgb
+
+extern "C" int lb_plan_flat(int32_t storage, const int64_t dims[3], int64_t n, int32_t sms, lb_flat_plan_t* out) {
+  using namespace lbgb;
+  if (!out || !dims || n < 2 || dims[2] != 1) return LB_E_INVAL;
+  for (int k = 0; k < 2; ++k)
+    if (dims[k] < 1 || dims[k] > (int64_t(1) << 30)) return LB_E_INVAL;
+  if (storage != LB_F64 && storage != LB_F32) return LB_E_UNSUPPORTED;
+  const bool fp64 = storage == LB_F64;
+  const int rows = fp64 ? k4_max_rows<double>() : k4_max_rows<float>();
+  const FlatSplit sp = split_run(dims[0], dims[1], n, rows, fp64, sms > 0 ? sms : k1_sm_count());
+  out->launches = sp.launches;
+  out->steps_first = launch_steps(n, sp.launches, 0);
+  out->steps_last = launch_steps(n, sp.launches, sp.launches - 1);
+  out->tile_rows = sp.bz;
+  out->max_rows = rows;
+  return LB_OK;
+}
