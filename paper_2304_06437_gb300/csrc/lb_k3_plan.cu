@@ -130,6 +130,9 @@ cudaError_t moment_run(lb_ctx* ctx, int64_t n) {
   cudaError_t e = cudaSuccess;
   if (m.v->leave && n % 2 == 0) {
     e = k1_step(ctx);
+    // the run ends by rebuilding the shell that this step read, so that launches
+    // recorded by a caller can be replayed: each time they find their shell
+    if (e == cudaSuccess) ctx->parity = 1 - ctx->parity;
     --n;
   }
   const int64_t launches = n - 1;
