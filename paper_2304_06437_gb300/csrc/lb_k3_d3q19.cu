@@ -1,6 +1,8 @@
 // lb_k3_d3q19.cu -- compiled tiles of the step in moment form for D3Q19.
 // Each entry: storage / arithmetic type, tile bx x by, TMA ring depth, nodes
-// per thread, CTAs per SM; and the brick cross-sections whose contexts can end a run.
+// per thread, CTAs per SM; and the brick cross-sections whose contexts can end a
+// run: all that are compiled, so that no batch, autotuner or requested brick takes a
+// context's runs away.
 #include "lb_k3_launch.cuh"
 
 namespace lbgb {
@@ -18,6 +20,9 @@ extern const LeaveVariant leave_variants_d3q19[] = {
     LeaveImpl<D3Q19, float, float, 64, 8, 3>::variant(LB_D3Q19, LB_F32),
     LeaveImpl<D3Q19, float, float, 32, 16, 3>::variant(LB_D3Q19, LB_F32),
     LeaveImpl<D3Q19, float, float, 32, 8, 2>::variant(LB_D3Q19, LB_F32),
+    LeaveImpl<D3Q19, float, float, 64, 7, 3>::variant(LB_D3Q19, LB_F32),
+    LeaveImpl<D3Q19, float, float, 64, 6, 3>::variant(LB_D3Q19, LB_F32),
+    LeaveImpl<D3Q19, float, float, 32, 14, 3>::variant(LB_D3Q19, LB_F32),
     LeaveImpl<D3Q19, double, double, 32, 8, 2>::variant(LB_D3Q19, LB_F64),
 };
 extern const int leave_n_variants_d3q19 = sizeof(leave_variants_d3q19) / sizeof(leave_variants_d3q19[0]);
