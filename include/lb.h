@@ -157,7 +157,9 @@ LB_API int lb_get_region(lb_ctx* ctx, const int64_t lo[3], const int64_t size[3]
  * fused scheme launches a pair of steps captured once as a CUDA graph (held
  * by the context until it is re-planned or destroyed); if the caller is
  * capturing the context stream, the steps are launched one by one and land
- * in the caller's graph.  Errors: LB_E_INVAL (n < 0, or n > 1 on a slab with
+ * in the caller's graph, which can be replayed where it holds an even number of
+ * steps, also between other calls, as long as those took an even number of
+ * steps in all since the capture.  Errors: LB_E_INVAL (n < 0, or n > 1 on a slab with
  * a link face), LB_E_CUDA (a launch failed). */
 LB_API int lb_step(lb_ctx* ctx, int64_t n);
 

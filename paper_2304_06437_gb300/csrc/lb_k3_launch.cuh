@@ -22,7 +22,9 @@ struct K3Variant {
 
 // The launches that end a run for contexts whose brick cross-section is
 // bx x by: the shell from coefficient set A, and the last step from set A to
-// the populations.
+// the populations.  The last step reads the shell that is not current and
+// writes the current one, so that a run of any length leaves the parity as it
+// was (recorded launches can be replayed, and a batch uploads no parities).
 struct LeaveVariant {
   int lattice, storage, bx, by;
   cudaError_t (*configure)();
@@ -138,14 +140,14 @@ struct LeaveImpl {
   }
 
   static cudaError_t shell(lb_ctx* ctx) {
-    K1Args<R> a = k1_make_args<R>(ctx, 1 - ctx->parity, ctx->parity);
+    K1Args<R> a = k1_make_args<R>(ctx, ctx->parity, 1 - ctx->parity);
     // the coefficients already hold the forcing: one instantiation serves both
     k1_bootstrap<L, S, R, BX, BY, false, true><<<k1_bootstrap_blocks(ctx->g, BX), 256, 0, ctx->stream>>>(a);
     return cudaGetLastError();
   }
 
   static cudaError_t leave(lb_ctx* ctx) {
-    K1Args<R> a = k1_make_args<R>(ctx, ctx->parity, 1 - ctx->parity);
+    K1Args<R> a = k1_make_args<R>(ctx, 1 - ctx->parity, ctx->parity);
     make_bounce_terms<L, R>(ctx->g, a.bb);
     const int grid = ctx->plan.nbx * ctx->plan.nby * ctx->plan.nbz;
     if (ctx->g.has_force)

@@ -155,9 +155,7 @@ cudaError_t moment_run(lb_ctx* ctx, int64_t n) {
     return e == cudaSuccess ? k1_bootstrap(ctx) : e;
   }
   if (e == cudaSuccess) e = m.lv->shell(ctx);
-  if (e == cudaSuccess) e = m.lv->leave(ctx);
-  if (e == cudaSuccess) ctx->parity = 1 - ctx->parity;
-  return e;
+  return e == cudaSuccess ? m.lv->leave(ctx) : e;
 }
 
 cudaError_t moment_run_beside(lb_ctx* ctx, int64_t n) {

@@ -12,8 +12,7 @@ pytestmark = pytest.mark.gpu
 
 # either side of the sizes that take another tile, and that run on their own in a batch
 DIMS = {"D2Q9": [(45, 31, 1), (300, 231, 1)], "D3Q19": [(37, 21, 13), (60, 56, 50)], "D3Q27": [(37, 21, 13), (60, 56, 50)]}
-FORMS = [(lat, st) for lat in DIMS for st in ("f64", "f32", "f16s", "bf16s")
-         if lat == "D2Q9" or st in ("f16s", "bf16s")]
+FORMS = [(lat, st) for lat in DIMS for st in ("f64", "f32", "f16s", "bf16s")]
 
 
 def _solver(lat, dims, storage, f0, stream=None):
