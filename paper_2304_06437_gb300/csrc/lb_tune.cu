@@ -39,7 +39,8 @@ TuneKey key_of(const lb_ctx* ctx) {
   return TuneKey{ctx->lattice, ctx->storage, g.nx, g.ny, nzc, kinds, g.has_force ? 1 : 0, 0, 0};
 }
 
-// time `steps` fused steps of one shape on a proxy; ms per node update x 1e6
+// time `steps` fused steps of one shape on a proxy, none of them in a run of
+// several; ms per node update x 1e6
 int time_variant(const lb_ctx* ctx, const void* v, int steps, double* ns_per_update, int32_t tile[3]) {
   const Geometry& g = ctx->g;
   int64_t dims[3] = {ctx->dims[0], ctx->dims[1], ctx->dims[2]};
@@ -55,15 +56,16 @@ int time_variant(const lb_ctx* ctx, const void* v, int steps, double* ns_per_upd
   int rc = lb_create(ctx->lattice, dims, ctx->tau_user, &ctx->bnd_user, &opt, &p);
   if (rc != LB_OK) return rc;
   rc = ctx_replan(p, v);
-  // runs on tiles of their own, from the first launch to the last, say nothing
-  // about the brick shape: time single steps
+  // runs step on tiles of their own and say nothing about the brick shape, which
+  // serves single steps, short calls and batches: time single steps
   p->flat_state = -1;
-  if (p->elem_bytes == 2) p->mr.state = -1;
+  p->mr.state = -1;
   const double u[3] = {0.01, 0.005, 0.0};
   if (rc == LB_OK) rc = lb_init_uniform(p, ctx->g.rho0, u);
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (rc == LB_OK && (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)) rc = LB_E_CUDA;
-  if (rc == LB_OK) rc = lb_step(p, 2);
+  // (a call of the timed kind, so that no first recording is timed)
+  if (rc == LB_OK) rc = lb_step(p, steps < kMomentMinSteps ? 2 : kMomentMinSteps);
   if (rc == LB_OK && cudaEventRecord(e0, p->stream) != cudaSuccess) rc = LB_E_CUDA;
   if (rc == LB_OK) rc = lb_step(p, steps);
   if (rc == LB_OK && cudaEventRecord(e1, p->stream) != cudaSuccess) rc = LB_E_CUDA;
