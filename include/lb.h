@@ -111,7 +111,8 @@ typedef struct {
   int64_t steps_done;
   int32_t tile[3];          /* brick (bx, by, bz) used by the fused scheme */
   uint64_t population_bytes; /* the one population array */
-  uint64_t aux_bytes;        /* shells (fused) or moment arrays (two-pass) */
+  uint64_t aux_bytes;        /* what else is allocated per node: shells and the memory of
+                                runs of several steps (fused) or moment arrays (two-pass) */
   uint64_t algorithmic_bytes_per_update; /* 2 q s: one read + one write per population */
   int32_t nodes_per_thread;  /* fused scheme: 1 scalar kernel, 2 paired FP32x2 kernel */
   int32_t tma_slots;         /* fused scheme: TMA ring depth */

@@ -847,7 +847,7 @@ int lb_info(const lb_ctx* ctx, lb_info_t* info) {
     info->tma_slots = ctx->plan.slots;
   }
   info->population_bytes = ctx->f_bytes;
-  info->aux_bytes = ctx->aux_bytes;
+  info->aux_bytes = ctx->f_alloc - ctx->f_bytes + (ctx->own_aux ? ctx->aux_bytes : 0);
   info->algorithmic_bytes_per_update = uint64_t(2) * ctx->g.q * ctx->elem_bytes;
   return LB_OK;
 }
