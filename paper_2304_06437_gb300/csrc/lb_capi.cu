@@ -207,13 +207,13 @@ int ctx_replan(lb_ctx* ctx, const void* variant, int bz) {
   drop_step_graph(ctx);
   drop_moment_run(ctx);
   const size_t aux_bytes = size_t(2) * size_t(p.parity_elems) * ctx->real_bytes;
-  void* aux = nullptr;
-  LB_TRY_CUDA(cudaMalloc(&aux, aux_bytes));
-  cudaError_t e = cudaMemsetAsync(aux, 0, aux_bytes, ctx->stream);
-  if (e != cudaSuccess) {
-    cudaFree(aux);
-    return cuda_status(e);
-  }
+  // the new shells take the old ones' place in the populations' allocation where
+  // they fit it (their contents follow from the populations), else they get an
+  // allocation of their own, and that place serves the runs of several steps alone
+  const size_t aux_at = align256(ctx->f_bytes);
+  const bool own = aux_bytes > ctx->f_alloc - aux_at;
+  void* aux = static_cast<char*>(ctx->f) + aux_at;
+  if (own) LB_TRY_CUDA(cudaMalloc(&aux, aux_bytes));
   const FusedPlan old_plan = ctx->plan;
   void* old_aux = ctx->aux;
   const size_t old_bytes = ctx->aux_bytes;
@@ -221,8 +221,9 @@ int ctx_replan(lb_ctx* ctx, const void* variant, int bz) {
   ctx->plan = p;
   ctx->aux = aux;
   ctx->aux_bytes = aux_bytes;
-  ctx->own_aux = true;
-  int rc = make_tensor_map(ctx);
+  ctx->own_aux = own;
+  int rc = cuda_status(cudaMemsetAsync(aux, 0, aux_bytes, ctx->stream));
+  if (rc == LB_OK) rc = make_tensor_map(ctx);
   if (rc == LB_OK) rc = cuda_status(k1_configure(ctx));
   if (rc == LB_OK) rc = after_state_change(ctx);  // rebuild the shell from the populations
   if (rc == LB_OK) rc = cuda_status(cudaStreamSynchronize(ctx->stream));
@@ -232,7 +233,9 @@ int ctx_replan(lb_ctx* ctx, const void* variant, int bz) {
     ctx->aux_bytes = old_bytes;
     ctx->own_aux = old_own;
     make_tensor_map(ctx);
-    cudaFree(aux);
+    if (!old_own) k1_bootstrap(ctx);
+    cudaStreamSynchronize(ctx->stream);
+    if (own) cudaFree(aux);
     return rc;
   }
   if (old_own) cudaFree(old_aux);

@@ -73,3 +73,17 @@ def test_info_after_a_batch(lb, lat, storage, dims):
         assert abs(before - _free() - _held(s)) <= SLACK
         assert _held(s) >= first
     assert abs(before - _free()) <= SLACK
+
+
+@pytest.mark.parametrize("lat,storage,dims", [("D3Q19", "f16s", (128, 128, 128)), ("D3Q27", "bf16s", (128, 128, 96)),
+                                              ("D3Q19", "bf16s", (96, 128, 112))])
+def test_shells_of_a_batch_take_the_room_there_is(lb, lat, storage, dims):
+    """The runs' memory lies idle where shells are read: a re-plan allocates
+    nothing beside it."""
+    with lb.Solver(lat, dims, 0.7, storage=storage) as s:
+        first, tile = _held(s), s.info()["tile"]
+        with lb.Batch([s]) as b:
+            b.step(1)
+            b.sync()
+            assert s.info()["tile"] != tile
+            assert _held(s) == first
