@@ -241,6 +241,17 @@ typedef struct {
 LB_API int lb_plan_fused(int32_t lattice, int32_t storage, const int64_t dims[3], const int32_t tile[3],
                          int32_t sms, lb_plan_t* out);
 
+/* Device memory of a fused context with the default brick (no device is
+ * touched): what lb_create() takes at the least, what it adds for runs of several
+ * steps (3D FP32 and FP64: where it can be had; 2D and 16-bit storage: where it
+ * is at most a sixteenth of the memory then free), and the shells that a batch
+ * may give it beside those.  The reductions' residual snapshot (12 bytes a
+ * node, lb_reduce) comes on top.  Errors: LB_E_INVAL, LB_E_UNSUPPORTED. */
+typedef struct {
+  uint64_t context_bytes, run_bytes, batch_bytes;
+} lb_context_bytes_t;
+LB_API int lb_plan_memory(int32_t lattice, int32_t storage, const int64_t dims[3], lb_context_bytes_t* out);
+
 /* How lb_step(n) divides a run of a 2D domain in FP64 or FP32 storage into
  * launches of several steps each (no device is touched): an even number of
  * launches, the first of them steps_first steps long and the last steps_last,

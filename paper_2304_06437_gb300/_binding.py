@@ -106,6 +106,10 @@ class lb_flat_plan_t(ctypes.Structure):
                 ("tile_rows", ctypes.c_int32), ("max_rows", ctypes.c_int32)]
 
 
+class lb_context_bytes_t(ctypes.Structure):
+    _fields_ = [("context_bytes", ctypes.c_uint64), ("run_bytes", ctypes.c_uint64), ("batch_bytes", ctypes.c_uint64)]
+
+
 class lb_batch_info_t(ctypes.Structure):
     _fields_ = [
         ("n_domains", ctypes.c_int32),
@@ -168,6 +172,7 @@ SIGNATURES = {
     "lb_plan_fused": (ctypes.c_int, [ctypes.c_int32, ctypes.c_int32, _i64p, _P(ctypes.c_int32), ctypes.c_int32,
                                      _P(lb_plan_t)]),
     "lb_plan_flat": (ctypes.c_int, [ctypes.c_int32, _i64p, ctypes.c_int64, ctypes.c_int32, _P(lb_flat_plan_t)]),
+    "lb_plan_memory": (ctypes.c_int, [ctypes.c_int32, ctypes.c_int32, _i64p, _P(lb_context_bytes_t)]),
     "lb_halo_bytes": (ctypes.c_int, [_vp, _i64p]),
     "lb_halo_pack": (ctypes.c_int, [_vp, ctypes.c_int32, _vp]),
     "lb_halo_unpack": (ctypes.c_int, [_vp, ctypes.c_int32, _vp]),

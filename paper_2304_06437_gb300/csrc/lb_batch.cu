@@ -192,14 +192,14 @@ int setup_class(lb_batch& b, lb_batch::Class& c) {
   return LB_OK;
 }
 
-// Re-plan a member for batched throughput: the first plain compiled shape (in
+// The brick that a batch gives a member: the first plain compiled shape (in
 // the planner's order) whose bricks pad the cross-section by at most 25 %, else
 // the least padded one; and, for sweeps of up to 256 planes, one brick per
 // column, so that small domains do not pay the pipeline fill (slots + 2
-// planes) and the z-shell of short bricks.  Bits are unchanged.
-int batch_replan(lb_ctx* x) {
+// planes) and the z-shell of short bricks (bz; 0: the planner's choice).
+const K1Variant* batch_variant(const Geometry& g, int storage, int* bz) {
   const void* vs[64];
-  const int nv = std::min(k1_variants_for(x->lattice, x->storage, vs, 64), 64);
+  const int nv = std::min(k1_variants_for(g.lattice, storage, vs, 64), 64);
   const K1Variant* pick = nullptr;
   const K1Variant* least = nullptr;
   double least_waste = 1e300;
@@ -208,26 +208,33 @@ int batch_replan(lb_ctx* x) {
     // plain shapes only: the decoupled-export and TMA-store alternatives
     // measure slower on the large domains they were tried on
     if (!v->batched || v->nxw != 0 || v->ts != 0) continue;
-    const double px = double((x->g.nx + v->bx - 1) / v->bx) * v->bx;
-    const double py = double((x->g.ny + v->by - 1) / v->by) * v->by;
-    const double waste = px * py / (double(x->g.nx) * double(x->g.ny));
+    const double px = double((g.nx + v->bx - 1) / v->bx) * v->bx;
+    const double py = double((g.ny + v->by - 1) / v->by) * v->by;
+    const double waste = px * py / (double(g.nx) * double(g.ny));
     if (!pick && waste <= 1.25) pick = v;
     if (waste < least_waste) {
       least_waste = waste;
       least = v;
     }
   }
-  if (!pick) pick = least;
-  if (!pick) return LB_E_UNSUPPORTED;
-  const int bz = x->g.nz <= 256 ? x->g.nz : 0;
+  *bz = g.nz <= 256 ? g.nz : 0;
+  return pick ? pick : least;
+}
+
+// Re-plan a member for batched throughput.  Bits are unchanged.
+int batch_replan(lb_ctx* x) {
+  int bz = 0;
+  const K1Variant* pick = batch_variant(x->g, x->storage, &bz);
   FusedPlan want;
-  if (!k1_plan_variant(x->g, pick, bz, &want)) return LB_E_UNSUPPORTED;
+  if (!pick || !k1_plan_variant(x->g, pick, bz, &want)) return LB_E_UNSUPPORTED;
   if (pick == k1_ctx_variant(x) && want.bz == x->plan.bz) return LB_OK;
   return ctx_replan(x, pick, bz);
 }
 
+constexpr int kShortestSplit = 64;  // planes
+
 // Split the bricks of a class that would not give each of its persistent
-// CTAs at least two: halving its members' sweep length (down to 64 planes)
+// CTAs at least two: halving its members' sweep length (down to kShortestSplit planes)
 // doubles their bricks, so that the static work list balances, at the price
 // of one more pipeline fill (slots + 2 planes) per added brick.  Bits are
 // unchanged.
@@ -245,8 +252,8 @@ int split_for_balance(lb_batch& b, lb_batch::Class& c) {
     bool changed = false;
     for (int m : c.members) {
       lb_ctx* x = b.ctxs[m];
-      if (x->plan.bz <= 64) continue;
-      const int rc = ctx_replan(x, c.v, std::max(64, (x->plan.bz + 1) / 2));
+      if (x->plan.bz <= kShortestSplit) continue;
+      const int rc = ctx_replan(x, c.v, std::max(kShortestSplit, (x->plan.bz + 1) / 2));
       if (rc != LB_OK) return rc;
       changed = true;
     }
@@ -346,6 +353,22 @@ int step_classes(lb_batch& b, std::vector<lb_batch::Class>& classes, cudaGraphEx
 }
 
 }  // namespace
+
+size_t batch_shell_bytes(const Geometry& g, int storage, size_t room) {
+  const size_t real_bytes = storage == LB_F64 ? 8 : 4;
+  int bz = 0;
+  const K1Variant* v = batch_variant(g, storage, &bz);
+  FusedPlan p;
+  if (!v || !k1_plan_variant(g, v, bz, &p)) return 0;
+  // as many bricks as split_for_balance() may make of a column
+  for (size_t most = 0;; p.bz = std::max(kShortestSplit, (p.bz + 1) / 2)) {
+    if (!k1_plan_variant(g, v, p.bz, &p)) return most;
+    const size_t bytes = size_t(2) * size_t(p.parity_elems) * real_bytes;
+    if (bytes > room) most = std::max(most, bytes);
+    if (p.bz <= kShortestSplit) return most;
+  }
+}
+
 }  // namespace lbgb
 
 using namespace lbgb;

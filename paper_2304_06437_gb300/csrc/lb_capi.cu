@@ -90,6 +90,40 @@ int make_tensor_map(lb_ctx* ctx) {
 
 size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
 
+// Bytes of a fused context's one allocation: the populations, from aux_at on the
+// shells (aux_bytes), and at the most what its runs of several steps need (both
+// at once: the shells are rebuilt at a run's end).  large: the runs of 2D domains
+// and of 16-bit ones need much more than the populations, and get it only where
+// that is little of what is free, so that large domains, and many of them, still
+// fit the card.
+struct Room {
+  size_t aux_at, least, most;
+  bool large;
+};
+Room room_of(const Geometry& g, int storage, size_t elem_bytes, size_t real_bytes, size_t aux_bytes) {
+  Room r;
+  r.aux_at = align256(size_t(g.q) * size_t(g.vol) * elem_bytes);
+  r.least = r.most = r.aux_at + aux_bytes;
+  r.large = g.d == 2 || elem_bytes == 2;
+  if (!g.zlink[0] && !g.zlink[1])
+    r.most = std::max(r.least, std::max(moment_scratch_elems(g, storage), flat_scratch_elems(g, storage)) * real_bytes);
+  return r;
+}
+
+// the internal axes of lb_create: 2D (x, y) -> (x, z)
+Geometry plan_geometry(int lattice, const int64_t dims[3]) {
+  Geometry g{};
+  g.lattice = lattice;
+  g.q = lattice_q(lattice);
+  g.d = lattice_d(lattice);
+  g.nx = int(dims[0]);
+  g.ny = g.d == 2 ? 1 : int(dims[1]);
+  g.nz = g.d == 2 ? int(dims[1]) : int(dims[2]);
+  g.pitch = (int64_t(g.nx) + 31) / 32 * 32;
+  g.vol = g.pitch * g.ny * g.nz;
+  return g;
+}
+
 // Host moment fields cross to and from the device through a buffer of at
 // most this size, in two halves: while the context stream converts the chunk
 // in one half, a copy stream moves the next (or previous) chunk through the
@@ -321,14 +355,7 @@ int lb_plan_fused(int32_t lattice, int32_t storage, const int64_t dims[3], const
   for (int k = 0; k < 3; ++k)
     if (dims[k] < 1 || dims[k] > (int64_t(1) << 30)) return LB_E_INVAL;
   if (d == 2 && dims[2] != 1) return LB_E_INVAL;
-  // the internal axes of lb_create: 2D (x, y) -> (x, z)
-  Geometry g{};
-  g.lattice = lattice;
-  g.q = q;
-  g.d = d;
-  g.nx = int(dims[0]);
-  g.ny = d == 2 ? 1 : int(dims[1]);
-  g.nz = d == 2 ? int(dims[1]) : int(dims[2]);
+  const Geometry g = plan_geometry(lattice, dims);
   FusedPlan p{};
   if (!k1_plan(g, storage, tile, &p, sms)) return LB_E_UNSUPPORTED;
   out->bx = p.bx;
@@ -343,6 +370,24 @@ int lb_plan_fused(int32_t lattice, int32_t storage, const int64_t dims[3], const
   out->export_warps = p.xwarps;
   out->shared_bytes = int64_t(p.smem_bytes);
   out->shell_elems_per_parity = p.sx_elems + p.sy_elems + p.sz_elems;
+  return LB_OK;
+}
+
+int lb_plan_memory(int32_t lattice, int32_t storage, const int64_t dims[3], lb_context_bytes_t* out) {
+  if (!out || !dims) return LB_E_INVAL;
+  if (lattice_q(lattice) < 0 || storage_bytes(storage) == 0) return LB_E_INVAL;
+  for (int k = 0; k < 3; ++k)
+    if (dims[k] < 1 || dims[k] > (int64_t(1) << 30)) return LB_E_INVAL;
+  if (lattice_d(lattice) == 2 && dims[2] != 1) return LB_E_INVAL;
+  const Geometry g = plan_geometry(lattice, dims);
+  const size_t real_bytes = storage == LB_F64 ? 8 : 4;
+  auto shells = [&](const FusedPlan& p) { return size_t(2) * size_t(p.parity_elems) * real_bytes; };
+  FusedPlan p{};
+  if (!k1_plan(g, storage, nullptr, &p, 0)) return LB_E_UNSUPPORTED;
+  const Room r = room_of(g, storage, storage_bytes(storage), real_bytes, shells(p));
+  out->context_bytes = r.least;
+  out->run_bytes = r.most - r.least;
+  out->batch_bytes = batch_shell_bytes(g, storage, r.least - r.aux_at);
   return LB_OK;
 }
 
@@ -459,33 +504,24 @@ int lb_create(int32_t lattice, const int64_t dims[3], double tau, const lb_bound
       ctx->aux_bytes = k0_aux_bytes(g, ctx->storage);
     }
     ctx->f_bytes = size_t(q) * size_t(g.vol) * ctx->elem_bytes;
-    // one allocation: the populations, then the shells or moment arrays; runs
-    // in moment form use both (the shells are rebuilt at their end)
-    const size_t aux_at = align256(ctx->f_bytes);
-    size_t want = aux_at + ctx->aux_bytes;
-    const size_t least = want;
-    if (ctx->scheme == LB_SCHEME_FUSED && !g.zlink[0] && !g.zlink[1]) {
-      const size_t runs = std::max(moment_scratch_elems(g, ctx->storage), flat_scratch_elems(g, ctx->storage)) *
-                          ctx->real_bytes;
-      // the runs of 2D domains and of 16-bit ones need much more than the
-      // populations: only where that is little of what is free, so that large
-      // domains, and many of them, still fit the card
-      size_t free_bytes = 0, total = 0;
-      const bool large = g.d == 2 || ctx->elem_bytes == 2;
-      if (runs > want && (!large || (cudaMemGetInfo(&free_bytes, &total) == cudaSuccess && free_bytes > want &&
-                                     (free_bytes - want) / 16 >= runs - want)))
-        want = runs;
-    }
+    // one allocation: the populations, then the shells or moment arrays
+    const bool fused = ctx->scheme == LB_SCHEME_FUSED;
+    const Room room = room_of(g, ctx->storage, ctx->elem_bytes, ctx->real_bytes, ctx->aux_bytes);
+    size_t want = room.least, free_bytes = 0, total = 0;
+    if (fused && room.most > want &&
+        (!room.large || (cudaMemGetInfo(&free_bytes, &total) == cudaSuccess && free_bytes > want &&
+                         (free_bytes - want) / 16 >= room.most - want)))
+      want = room.most;
     cudaError_t e = cudaMalloc(&ctx->f, want);
-    if (e == cudaErrorMemoryAllocation && want > least) {
+    if (e == cudaErrorMemoryAllocation && want > room.least) {
       cudaGetLastError();
-      want = least;
+      want = room.least;
       e = cudaMalloc(&ctx->f, want);
     }
     if (e != cudaSuccess) { rc = cuda_status(e); break; }
     ctx->f_alloc = want;
     if (ctx->aux_bytes) {
-      ctx->aux = static_cast<char*>(ctx->f) + aux_at;
+      ctx->aux = static_cast<char*>(ctx->f) + room.aux_at;
       e = cudaMemsetAsync(ctx->aux, 0, ctx->aux_bytes, ctx->stream);
       if (e != cudaSuccess) { rc = cuda_status(e); break; }
     }

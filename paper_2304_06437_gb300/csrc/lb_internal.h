@@ -175,6 +175,11 @@ bool flat_plan(lb_ctx* ctx);
 // n >= 2 steps of a planned context; beside: other runs share the device
 cudaError_t flat_run(lb_ctx* ctx, int64_t n, bool beside = false);
 
+// ---- batches (lb_batch.cu)
+// bytes of the shells that a batch may give a context of its own, where they
+// don't fit the room of those it was created with (0: they do)
+size_t batch_shell_bytes(const Geometry& g, int storage, size_t room);
+
 // ---- state conversion, readout and reductions (lb_aux.cu)
 cudaError_t aux_set_populations(lb_ctx* ctx, const double* f_dev);
 cudaError_t aux_get_populations(lb_ctx* ctx, double* f_dev);

@@ -36,7 +36,7 @@ from typing import Callable, List, Optional
 import numpy as np
 
 from ._binding import LB_E_NOMEM, LBError
-from .solver import Batch, Solver
+from .solver import Batch, Solver, context_bytes
 
 
 @dataclasses.dataclass
@@ -62,17 +62,12 @@ class Request:
     u: Optional[np.ndarray] = None
 
 
-Q_OF = {"D2Q9": 9, "D3Q19": 19, "D3Q27": 27}
-BYTES_OF = {"f64": 8, "f32": 4, "f16s": 2, "bf16s": 2}
-
-
 def footprint_bytes(req: Request) -> int:
-    """Device bytes a request holds while resident: the population array,
-    the brick shells (bounded by a quarter of the populations for the
-    compiled brick shapes), the FP32 residual snapshot of u and slack."""
+    """Device bytes a request may hold while resident: its context with the
+    memory of runs of several steps, the shells that a batch may give it, the
+    FP32 residual snapshot of u and slack."""
     n = int(np.prod(req.dims))
-    pop = Q_OF[req.lattice] * BYTES_OF[req.storage] * n
-    return int(1.25 * pop + 12 * n + (4 << 20))
+    return sum(context_bytes(req.lattice, req.dims, req.storage).values()) + 12 * n + (4 << 20)
 
 
 class Server:

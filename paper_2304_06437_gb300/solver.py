@@ -492,6 +492,19 @@ def fused_plan(lattice, dims, storage="f32", tile=None, sms=0) -> dict:
     return {name: getattr(p, name) for name, _ in p._fields_}
 
 
+def context_bytes(lattice, dims, storage="f32") -> dict:
+    """Device memory that a fused context may take (lb_plan_memory; no device
+    is touched)."""
+    lib = B.load()
+    lid = B.LATTICES[lattice] if isinstance(lattice, str) else int(lattice)
+    st = B.STORAGES[storage] if isinstance(storage, str) else int(storage)
+    dims = list(dims) + [1] * (3 - len(dims))
+    p = B.lb_context_bytes_t()
+    B.check(lib.lb_plan_memory(lid, st, (ctypes.c_int64 * 3)(*[int(v) for v in dims[:3]]), ctypes.byref(p)),
+            "lb_plan_memory")
+    return {name: getattr(p, name) for name, _ in p._fields_}
+
+
 def memory_plan(lattice, bytes_per_value=4) -> dict:
     lib = B.load()
     lid = B.LATTICES[lattice] if isinstance(lattice, str) else int(lattice)

@@ -87,3 +87,30 @@ def test_shells_of_a_batch_take_the_room_there_is(lb, lat, storage, dims):
             b.sync()
             assert s.info()["tile"] != tile
             assert _held(s) == first
+
+
+@pytest.mark.parametrize("lat,storage,dims", [f for f in FORMS if f[1] != "two_pass"] +
+                         [("D3Q19", "f32", (66, 130, 192)), ("D3Q27", "f16s", (100, 100, 100))])
+def test_a_served_request_holds_no_more_than_its_footprint(lb, lat, storage, dims):
+    from paper_2304_06437_gb300 import serve
+    from paper_2304_06437_gb300.solver import context_bytes
+
+    def use(s):
+        with lb.Batch([s]) as b:
+            b.step(6)
+            b.step(1)
+            b.sync()
+        return _free()
+
+    with lb.Solver(lat, dims, 0.7, storage=storage) as s:
+        use(s)
+    before = _free()
+    # but the snapshot of u, which comes from a pool that contexts share
+    foot = serve.footprint_bytes(serve.Request(0, 0.0, lat, dims, 0.7, [0] * 6, storage=storage)) - 12 * np.prod(dims)
+    with lb.Solver(lat, dims, 0.7, storage=storage) as s:
+        plan = context_bytes(lat, dims, storage)
+        assert _held(s) == plan["context_bytes"] + plan["run_bytes"]
+        held = before - use(s)
+        assert _held(s) <= sum(plan.values()) <= foot
+    assert held <= foot + SLACK
+    assert foot <= 1.5 * held + SLACK
