@@ -384,6 +384,11 @@ LB_API int lb_batch_reduce(lb_batch* b, int32_t want_residual, double* out);
 LB_API int lb_batch_sync(lb_batch* b);
 LB_API int lb_batch_info(const lb_batch* b, lb_batch_info_t* info);
 
+/* The members that calls of four or more steps run on their own: writes up to
+ * cap of their indices (in the order given to lb_batch_create, the largest
+ * first) to members (may be NULL) and returns their number, or LB_E_INVAL. */
+LB_API int lb_batch_alone(const lb_batch* b, int32_t* members, int32_t cap);
+
 /* Frees the batch (not its contexts).  NULL is allowed. */
 LB_API void lb_batch_destroy(lb_batch* b);
 

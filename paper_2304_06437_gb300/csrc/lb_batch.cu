@@ -601,6 +601,12 @@ int lb_batch_info(const lb_batch* b, lb_batch_info_t* info) {
   return LB_OK;
 }
 
+int lb_batch_alone(const lb_batch* b, int32_t* members, int32_t cap) {
+  if (!b || cap < 0) return LB_E_INVAL;
+  for (size_t k = 0; members && k < b->runs.size() && k < size_t(cap); ++k) members[k] = b->runs[k];
+  return int(b->runs.size());
+}
+
 void lb_batch_destroy(lb_batch* b) {
   if (!b) return;
   DevGuard guard(b->device);

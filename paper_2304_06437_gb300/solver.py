@@ -265,6 +265,13 @@ class Batch:
         B.check(self._lib.lb_batch_info(self._b, ctypes.byref(inf)), "lb_batch_info")
         return {name: getattr(inf, name) for name, _ in inf._fields_}
 
+    def alone(self) -> list:
+        """Indices of the members that calls of four or more steps run on
+        their own, the largest first (lb_batch_alone)."""
+        idx = (ctypes.c_int32 * len(self.solvers))()
+        n = B.check(self._lib.lb_batch_alone(self._b, idx, len(self.solvers)), "lb_batch_alone")
+        return list(idx[:n])
+
     def close(self):
         if getattr(self, "_b", None) and self._b.value:
             self._lib.lb_batch_destroy(self._b)
