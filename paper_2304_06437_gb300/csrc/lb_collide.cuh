@@ -77,9 +77,6 @@ struct Phys {
   R cs2;     // 1/3 rounded to R
   // products of the constants above, formed once in FP64 on the host
   R c15rho0, c15om1, c3rho0, c45rho0, c45om1, c9rho0, c9om1, c3g, c9g;
-  // negated constants, for packed arithmetic (lb_pair.cuh), whose operands
-  // carry no sign
-  R n_rho0, n_inv_rho0, n_cs2, n15rho0, n15om1, n3g;
 };
 
 LB_DEV float fma_r(float a, float b, float c) { return fmaf(a, b, c); }
@@ -356,6 +353,29 @@ LB_DEV void post_all(const Coef<R>& k, R (&out)[L::Q]) {
     out[a] = fma_r(w, even, wodd);
     out[b] = fma_r(w, even, -wodd);
   });
+}
+
+// populations -> coefficients of the post-collision set
+template <class L, bool FORCE, class R>
+LB_DEV void moments_coeffs(const R (&f)[L::Q], const Phys<R>& ph, Coef<R>& k) {
+  Mom<R> m;
+  moments<L, R, FORCE>(f, ph, m);
+  coeffs<L, R, FORCE>(m, ph, k);
+}
+
+// both members of a velocity pair {a, opp(a)} whose first non-zero component is
+// +1 for a
+template <class L>
+LB_HD constexpr int leading_sign(int a) {
+  return L::cx(a) != 0 ? L::cx(a) : (L::cy(a) != 0 ? L::cy(a) : L::cz(a));
+}
+template <class L, int a, class R>
+LB_DEV void post_pair(const Coef<R>& k, R& fa, R& fo) {
+  constexpr R w = R(weight<L>(a));
+  R even, wodd;
+  post_parts<L, R, a>(k, even, wodd);
+  fa = fma_r(w, even, wodd);
+  fo = fma_r(w, even, -wodd);
 }
 
 // full regularized collision of one node: ft -> ft*

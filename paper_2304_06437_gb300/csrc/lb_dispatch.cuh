@@ -59,12 +59,6 @@ Phys<R> make_phys(const Geometry& g) {
   p.c9om1 = R(9.0 * om1);
   p.c3g = R(3.0 * gg);
   p.c9g = R(9.0 * gg);
-  p.n_rho0 = R(-g.rho0);
-  p.n_inv_rho0 = R(-1.0 / g.rho0);
-  p.n_cs2 = R(-1.0 / 3.0);
-  p.n15rho0 = R(-1.5 * r0);
-  p.n15om1 = R(-1.5 * om1);
-  p.n3g = R(-3.0 * gg);
   return p;
 }
 

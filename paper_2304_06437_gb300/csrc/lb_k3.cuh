@@ -40,19 +40,18 @@
 //
 // Layout of a launch: a CTA owns a tile of bx x by nodes and sweeps bz planes.
 // TMA streams the tile's coefficients plane by plane into a ring of shared
-// slots; each node thread evaluates the post-collision set of its node, or of
-// the two nodes x and x + 1 (NPT = 2: packed FP32x2 arithmetic, lb_pair.cuh),
-// and puts the laterally moving populations into a shared window (three
-// buffers).  Halo warps fill the one-node ring around the tile, from loads
-// issued a plane ahead: with the populations that enter from the neighbouring
-// tiles, or, where the tile borders an x or y wall, with the bounce-back
-// values of the wall's own nodes, so that the node warps gather without any
-// test for walls.  One split barrier per plane: a warp arrives once its part
-// of a window is written and waits when it needs the whole.
+// slots; each node thread evaluates the post-collision set of its node and puts
+// the laterally moving populations into a shared window (three buffers).  Halo
+// warps fill the one-node ring around the tile, from loads issued a plane ahead:
+// with the populations that enter from the neighbouring tiles, or, where the
+// tile borders an x or y wall, with the bounce-back values of the wall's own
+// nodes, so that the node warps gather without any test for walls.  One split
+// barrier per plane: a warp arrives once its part of a window is written and
+// waits when it needs the whole.  (Two nodes a thread in packed FP32x2
+// arithmetic measured slower.)
 #pragma once
 
 #include "lb_k1.cuh"
-#include "lb_pair.cuh"
 
 namespace lbgb {
 
@@ -66,10 +65,9 @@ LB_HD inline int64_t k3_edge(int side, int tI, int ntx, int64_t rows, int64_t r)
   return (int64_t(side) * ntx + tI) * rows + r;
 }
 
-// V: the type of a thread's values, R or f32x2 (two nodes)
-template <class R, class V>
+template <class R>
 struct K3Args {
-  Phys<V> ph;
+  Phys<R> ph;
   int nx, ny, nz;
   int64_t pitch, vol;
   int per[3];
@@ -92,36 +90,30 @@ LB_HD constexpr int nonlateral_dir() {
   return -1;
 }
 
-template <class L, class R, int BX, int BY, int NS, int NPT, int MINB>
+template <class L, class R, int BX, int BY, int NS, int MINB>
 struct K3Shape {
-  using V = typename std::conditional<NPT == 2, f32x2, R>::type;
   static constexpr int Q = L::Q;
   static constexpr int NC = n_coef<L>();
   static constexpr int NYF = count_dirs<L>(1, 1);
   static constexpr int PY = NYF > 0 ? 1 : 0;
-  static constexpr int HB = BX / NPT;      // node threads per row
-  static constexpr int NTM = HB * BY;      // node threads
+  static constexpr int NTM = BX * BY;      // node threads
   static constexpr int WY = BY + 2 * PY;   // window rows
   // Window of one direction: rows of the tile and its ring.  A direction with
   // cx = 0 needs no ring along x: rows of BX values.  The others have rows of
-  // BX + 2, and with two nodes per thread the even and the odd nodes of a row
-  // apart (E(0) .. E(HB), then O(-1) .. O(HB - 1)), so that a thread's pair,
-  // shifted by one node, is two loads of consecutive lanes.
+  // BX + 2, column xl of the tile (-1 .. BX) at xl + 1.
   LB_HD static constexpr int row(int a) { return L::cx(a) == 0 ? BX : BX + 2; }
+  // position of the tile's column xl in a row of a moving direction
+  LB_HD static constexpr int col(int xl) { return xl + 1; }
   LB_HD static constexpr int off(int a) {
     int n = 0;
     for (int b = 0; b < a; ++b)
       if (is_lateral<L>(b)) n += WY * row(b);
     return n;
   }
-  // position of the tile's column xl (-1 .. BX) in a row of a moving direction
-  LB_HD static constexpr int col(int xl) {
-    return NPT == 2 ? ((xl & 1) ? HB + 1 + (xl + 1) / 2 : xl / 2) : xl + 1;
-  }
-  // halo threads: south and north rows (one per node thread column), then the
+  // halo threads: south and north rows (one per column), then the
   // west and east columns with the corners, each column in warps of its own
   // (a warp of two faces runs both in turn, and is then what the others wait for)
-  static constexpr int HROW = NYF > 0 ? 2 * HB : 0;
+  static constexpr int HROW = NYF > 0 ? 2 * BX : 0;
   static constexpr int HCOL = NYF > 0 ? (WY + 31) / 32 * 32 : 16;
   static constexpr int HWARPS = (HROW + 2 * HCOL) / 32;
   static constexpr int NT = NTM + 32 * HWARPS;
@@ -131,48 +123,35 @@ struct K3Shape {
   static constexpr size_t OFF_WIN = align128(size_t(NS) * SLOTN * sizeof(R));
   static constexpr size_t SMEM_CAP = (size_t(228) * 1024) / MINB - 1024;
   static constexpr int NW = 3;  // window buffers
-  // the halo threads' coefficients, HD planes deep (rows: V, columns: R)
+  // the halo threads' coefficients, HD planes deep
   static constexpr int HD = 4;
-  static constexpr size_t HSTAGE = size_t(NC) * (HROW * sizeof(V) + 2 * HCOL * sizeof(R));
+  static constexpr size_t HSTAGE = size_t(NC) * (HROW + 2 * HCOL) * sizeof(R);
   static constexpr size_t OFF_HALO = OFF_WIN + NW * WIN;
   static constexpr size_t OFF_BAR = align128(OFF_HALO + HD * HSTAGE);
   static constexpr size_t SMEM = OFF_BAR + align128((NS + NW) * sizeof(uint64_t));
   static_assert(SMEM <= SMEM_CAP, "shared memory of the shape exceeds its share of the SM");
   static_assert(NTM % 32 == 0 && NT <= 1024, "whole warps");
   static_assert(BY == 1 || NYF > 0, "a 2D tile has one internal row");
-  static_assert(NPT == 1 || (std::is_same<R, float>::value && BX % 2 == 0), "pairs are FP32");
   static_assert(HROW % 32 == 0, "a halo warp holds rows or columns, not both");
 };
 
-// lane l of a thread's value
-template <class R>
-LB_DEV R& lane_of(R& v, int) { return v; }
-LB_DEV float& lane_of(f32x2& v, int l) { return l == 0 ? v.x : v.y; }
-
-// lane l's coefficients as one record (16- or 8-byte stores)
-template <class L, class R, class V>
-LB_DEV void put_record(Coef<V>& k, R* e, int l) {
+// a node's coefficients as one record (16- or 8-byte stores)
+template <class L, class R>
+LB_DEV void put_record(Coef<R>& k, R* e) {
   using R2 = typename std::conditional<sizeof(R) == 4, float2, double2>::type;
   R rec[n_coef<L>()];
-  each_coef<L, V>(k, [&](auto I, V& v) { rec[decltype(I)::value] = l == 0 ? lane_of(v, 0) : lane_of(v, 1); });
+  each_coef<L, R>(k, [&](auto I, R& v) { rec[decltype(I)::value] = v; });
 #pragma unroll
   for (int i = 0; i < n_coef<L>(); i += 2) reinterpret_cast<R2*>(e)[i / 2] = R2{rec[i], rec[i + 1]};
 }
 
-template <class S, class R>
-LB_DEV R round_value(R v) { return round_to_storage<S, R>(v); }
-template <class S>
-LB_DEV f32x2 round_value(f32x2 v) { return round_pair<S>(v); }
-
 // One step of one brick (tile column tI, tJ, sweep tK): src -> dst, or (POP)
 // src -> populations, the last step of a run whose set A lies behind them.
-template <class L, class S, class R, int BX, int BY, int NS, int NPT, bool FORCE, int MINB, bool POP>
-__device__ __forceinline__ void k3_brick(
-    const CUtensorMap* tmap_p, const K3Args<R, typename K3Shape<L, R, BX, BY, NS, NPT, MINB>::V>& args, const int tI,
-    const int tJ, const int tK) {
-  using Sh = K3Shape<L, R, BX, BY, NS, NPT, MINB>;
-  using V = typename Sh::V;
-  constexpr int Q = L::Q, NC = Sh::NC, NTM = Sh::NTM, NYF = Sh::NYF, PY = Sh::PY, HB = Sh::HB;
+template <class L, class S, class R, int BX, int BY, int NS, bool FORCE, int MINB, bool POP>
+__device__ __forceinline__ void k3_brick(const CUtensorMap* tmap_p, const K3Args<R>& args, const int tI, const int tJ,
+                                         const int tK) {
+  using Sh = K3Shape<L, R, BX, BY, NS, MINB>;
+  constexpr int Q = L::Q, NC = Sh::NC, NTM = Sh::NTM, NYF = Sh::NYF, PY = Sh::PY;
   constexpr int WY = Sh::WY, HROW = Sh::HROW, NW = Sh::NW;
   constexpr int RM = BX + 2;  // row of a moving direction
   constexpr int WSTRIDE = int(Sh::WIN / sizeof(R));
@@ -253,21 +232,18 @@ __device__ __forceinline__ void k3_brick(
     using i1 = std::integral_constant<int, 1>;
     using im = std::integral_constant<int, -1>;
 
-    // T: the type of this thread's values (rows: V, columns: R); face, kind,
-    // the column xl and window row r of the ring cell (kind 2: the node's own
-    // column, and r the row beyond the wall for rows); the node (kind 2); its
-    // coefficients in plane 0 (rows: in the fields, columns: an edge record)
-    auto run = [&](auto tag, auto col_tag, const int face, const int kind, const int xl, const int r, const int sx,
+    // face, kind, the column xl and window row r of the ring cell (kind 2: the
+    // node's own column, and r the row beyond the wall for rows); the node (kind
+    // 2); its coefficients in plane 0 (rows: in the fields, columns: an edge record)
+    auto run = [&](auto col_tag, const int face, const int kind, const int xl, const int r, const int sx,
                    const int sy, const R* const p0) {
-      using T = typename decltype(tag)::type;
       constexpr bool COL = decltype(col_tag)::value;
-      constexpr bool ROW = !COL && NPT == 2;  // two nodes
       // plane zb + p is copied to stage p % HD of this thread's own shared
       // memory, HD - 2 planes ahead (a plane's time is about a loaded memory
       // latency: with loads one plane ahead the whole CTA waited for them)
       constexpr int HD = Sh::HD, HT = COL ? 2 * Sh::HCOL : HROW;
       using R2 = typename std::conditional<sizeof(R) == 4, float2, double2>::type;
-      unsigned char* const stage0 = smem + Sh::OFF_HALO + (COL ? size_t(HD) * NC * HROW * sizeof(V) : 0);
+      unsigned char* const stage0 = smem + Sh::OFF_HALO + (COL ? size_t(HD) * NC * HROW * sizeof(R) : 0);
       const int ht = COL ? hid - HROW : hid;
       auto fetch = [&](int p) {
         const int z = zb + p;
@@ -280,16 +256,16 @@ __device__ __forceinline__ void k3_brick(
           } else {
             const char* g = reinterpret_cast<const char*>(p0 + plane * zwrap(z));
             const uint32_t v32 = args.vol32;
-            T* h = reinterpret_cast<T*>(stage0) + (p % HD) * NC * HT + ht;
+            R* h = reinterpret_cast<R*>(stage0) + (p % HD) * NC * HT + ht;
 #pragma unroll
             for (int i = 0; i < NC; ++i)
-              cp_async<sizeof(T)>(h + i * HT, g + uint64_t(v32) * uint32_t(i * 32 * sizeof(R)));
+              cp_async<sizeof(R)>(h + i * HT, g + uint64_t(v32) * uint32_t(i * 32 * sizeof(R)));
           }
         }
         cp_async_commit();
       };
       auto coef_of = [&](int p) {
-        T h[NC];
+        R h[NC];
         if constexpr (COL) {
           const R2* hs = reinterpret_cast<const R2*>(stage0) + (p % HD) * (NC / 2) * HT + ht;
 #pragma unroll
@@ -299,83 +275,60 @@ __device__ __forceinline__ void k3_brick(
             h[i + 1] = v.y;
           }
         } else {
-          const T* hs = reinterpret_cast<const T*>(stage0) + (p % HD) * NC * HT + ht;
+          const R* hs = reinterpret_cast<const R*>(stage0) + (p % HD) * NC * HT + ht;
 #pragma unroll
           for (int i = 0; i < NC; ++i) h[i] = hs[i * HT];
         }
-        Coef<T> k;
-        each_coef<L, T>(k, [&](auto I, T& v) { v = h[decltype(I)::value]; });
+        Coef<R> k;
+        each_coef<L, R>(k, [&](auto I, R& v) { v = h[decltype(I)::value]; });
         return k;
       };
       // bounce-back values of the node's descending links, for the next window
-      T held[Q];
+      R held[Q];
 #pragma unroll
-      for (int a = 0; a < Q; ++a) held[a] = T(R(0));
-      // x sides a lane touches: bit 0 low, bit 1 high
-      auto x_walls = [&](int l) {
-        const int x = sx + l;
-        return args.per[0] ? 0 : (x == 0 ? 1 : 0) | (x == nx - 1 ? 2 : 0);
-      };
+      for (int a = 0; a < Q; ++a) held[a] = R(0);
+      // sides the node touches: bit 0 low, bit 1 high
       const int y_walls = args.per[1] ? 0 : (sy == 0 ? 1 : 0) | (sy == ny - 1 ? 2 : 0);
-      const int xw0 = x_walls(0), xw1 = ROW ? x_walls(1) : 0;
+      const int x_walls = args.per[0] ? 0 : (sx == 0 ? 1 : 0) | (sx == nx - 1 ? 2 : 0);
 
       auto produce = [&](int p, auto AX, auto SG) {
         constexpr int ax = decltype(AX)::value, sg = decltype(SG)::value;
         R* win = win0 + (p % NW) * WSTRIDE;
         if (kind == 1) {
-          const Coef<T> k = coef_of(p);
+          const Coef<R> k = coef_of(p);
           static_for<0, Q>([&](auto A_) {
             constexpr int a = decltype(A_)::value;
             if constexpr (comp<L>(ax, a) == sg) {
-              T v = post_v<L, a>(k);
+              R v = post<L, R, a>(k);
               R* w = win + Sh::off(a) + r * Sh::row(a);
-              if constexpr (L::cx(a) == 0) {
-                *reinterpret_cast<T*>(w + xl) = v;
-              } else if constexpr (ROW) {
-                w[xl / 2] = lane_of(v, 0);
-                if (xl + 1 < bxa) w[HB + 1 + xl / 2 + 1] = lane_of(v, 1);
-              } else {
-                w[Sh::col(xl)] = v;
-              }
+              if constexpr (L::cx(a) == 0) w[xl] = v;
+              else w[Sh::col(xl)] = v;
             }
           });
         } else if (kind == 2) {
-          const Coef<T> k = coef_of(p), kn = coef_of(p + 1);
+          const Coef<R> k = coef_of(p), kn = coef_of(p + 1);
           static_for<0, Q>([&](auto A_) {
             constexpr int a = decltype(A_)::value;
             constexpr int cx = L::cx(a), cy = L::cy(a), cz = L::cz(a);
             if constexpr (comp<L>(ax, a) == sg) {
               // the link of this node through the wall: the node's own opposite
               // population of the destination plane, c + cz
-              auto bounce = [&](const Coef<T>& kk) {
-                T v = post_v<L, L::opp(a)>(kk);
-                auto add = [&](int l, int xw) {
-                  int cb = 0;
-                  if constexpr (cx == 1) cb |= xw & 1;
-                  if constexpr (cx == -1) cb |= xw >> 1;
-                  if constexpr (cy == 1) cb |= (y_walls & 1) << 1;
-                  if constexpr (cy == -1) cb |= y_walls & 2;
-                  lane_of(v, l) = lane_of(v, l) + args.bb[a][cb];
-                };
-                add(0, xw0);
-                if constexpr (ROW) add(1, xw1);
-                return v;
+              auto bounce = [&](const Coef<R>& kk) {
+                int cb = 0;
+                if constexpr (cx == 1) cb |= x_walls & 1;
+                if constexpr (cx == -1) cb |= x_walls >> 1;
+                if constexpr (cy == 1) cb |= (y_walls & 1) << 1;
+                if constexpr (cy == -1) cb |= y_walls & 2;
+                return post<L, R, L::opp(a)>(kk) + args.bb[a][cb];
               };
-              T v;
+              R v;
               if constexpr (cz == 0) v = bounce(k);
               else if constexpr (cz == 1) v = bounce(kn);
               else v = held[a];
               if constexpr (cz == -1) held[a] = bounce(k);
               R* w = win + Sh::off(a) + (ax == 1 ? r : r - cy) * Sh::row(a);
-              if constexpr (cx == 0) {
-                *reinterpret_cast<T*>(w + xl) = v;
-              } else if constexpr (ROW) {
-                // cells xl - cx and xl + 1 - cx
-                w[cx == 1 ? HB + 1 + xl / 2 : HB + 2 + xl / 2] = lane_of(v, 0);
-                if (xl + 1 < bxa) w[cx == 1 ? xl / 2 : xl / 2 + 1] = lane_of(v, 1);
-              } else {
-                w[Sh::col(xl - cx)] = v;
-              }
+              if constexpr (cx == 0) w[xl] = v;
+              else w[Sh::col(xl - cx)] = v;
             }
           });
         }
@@ -398,14 +351,14 @@ __device__ __forceinline__ void k3_brick(
     };
 
     if (hid < HROW) {
-      const int face = hid < HB ? 2 : 3;
-      const int xl = (hid % HB) * NPT;
+      const int face = hid < BX ? 2 : 3;
+      const int xl = hid % BX;
       const bool wall = face == 2 ? wallS : wallN;
       int sy = face == 2 ? y0 - 1 : y0 + bya;
       if (wall) sy = face == 2 ? y0 : y0 + bya - 1;  // the wall's own row
       else sy = sy < 0 ? sy + ny : (sy >= ny ? sy - ny : sy);
-      run(type_tag<V>{}, std::false_type{}, face, xl < bxa ? (wall ? 2 : 1) : 0, xl, face == 2 ? 0 : bya + 1, x0 + xl,
-          sy, args.src + (x0 + xl) + args.pitch * sy);
+      run(std::false_type{}, face, xl < bxa ? (wall ? 2 : 1) : 0, xl, face == 2 ? 0 : bya + 1, x0 + xl, sy,
+          args.src + (x0 + xl) + args.pitch * sy);
     } else {
       const int k = hid - HROW;
       const int r = k % Sh::HCOL, yl = r - PY;
@@ -430,7 +383,7 @@ __device__ __forceinline__ void k3_brick(
       if (kind == 0) sy = 0;
       // the ring column, or at a wall the column of the node itself
       const int xl = face == 0 ? (wall ? 0 : -1) : (wall ? bxa - 1 : bxa);
-      run(type_tag<R>{}, std::true_type{}, face, kind, xl, r, x0 + xl, sy,
+      run(std::true_type{}, face, kind, xl, r, x0 + xl, sy,
           args.esrc + k3_edge(side, tc, args.ntx, int64_t(ny) * nz, sy) * NC);
     }
     if (dead) atomicExch(args.status, LB_E_TIMEOUT);
@@ -438,65 +391,49 @@ __device__ __forceinline__ void k3_brick(
   }
 
   // -------------------------------------------------------------- node warps
-  const int i = tid % HB, ty = tid / HB;
-  const int x = x0 + NPT * i, y = y0 + ty;
-  const bool active = NPT * i < bxa && ty < bya;
-  const bool act1 = NPT * i + 1 < bxa;  // the pair's second node
+  const int i = tid % BX, ty = tid / BX;
+  const int x = x0 + i, y = y0 + ty;
+  const bool active = i < bxa && ty < bya;
   const bool z_walls = !args.per[2];
   // this thread's place in the rows of the two kinds of directions
-  const int b0 = (ty + PY) * BX + NPT * i;
+  const int b0 = (ty + PY) * BX + i;
   const int bm = (ty + PY) * RM + i;
   R* const out0 = args.dst + x + args.pitch * y;
-  // edge records this thread writes: of the tile's first column (its node 0)
-  // and last column (node eastl)
-  const bool west = i == 0, east = NPT * i < bxa && NPT * (i + 1) >= bxa;
-  const int eastl = bxa - 1 - NPT * i;
+  // edge records this thread writes: of the tile's first and last columns
+  const bool west = i == 0, east = i < bxa && i + 1 >= bxa;
   R* const edge0 = args.edst + k3_edge(west ? 0 : 1, tI, args.ntx, int64_t(ny) * nz, y) * NC;
   constexpr int zm = nonlateral_dir<L, -1>(), zp = nonlateral_dir<L, 1>();
 
-  auto put = [&](R* win, auto A_, V v) {
+  auto put = [&](R* win, auto A_, R v) {
     constexpr int a = decltype(A_)::value;
-    if constexpr (L::cx(a) == 0) {
-      *reinterpret_cast<V*>(win + Sh::off(a) + b0) = v;
-    } else if constexpr (NPT == 2) {
-      win[Sh::off(a) + bm] = lane_of(v, 0);
-      if (act1) win[Sh::off(a) + bm + HB + 2] = lane_of(v, 1);
-    } else {
-      win[Sh::off(a) + bm + 1] = lane_of(v, 0);
-    }
+    if constexpr (L::cx(a) == 0) win[Sh::off(a) + b0] = v;
+    else win[Sh::off(a) + bm + 1] = v;
   };
-  // the values of direction a at the thread's nodes shifted by (-dx, -dy)
-  auto get = [&](const R* win, auto A_, auto DX, auto DY) -> V {
+  // the value of direction a at the thread's node shifted by (-dx, -dy)
+  auto get = [&](const R* win, auto A_, auto DX, auto DY) -> R {
     constexpr int a = decltype(A_)::value, dx = decltype(DX)::value, dy = decltype(DY)::value;
     if constexpr (L::cx(a) == 0) {
-      return *reinterpret_cast<const V*>(win + Sh::off(a) + b0 - dy * BX);
+      return win[Sh::off(a) + b0 - dy * BX];
     } else {
       const R* w = win + Sh::off(a) + bm - dy * RM;
-      V v;
-      if constexpr (NPT == 2) {
-        lane_of(v, 0) = w[dx == 0 ? 0 : (dx == 1 ? HB + 1 : HB + 2)];
-        lane_of(v, 1) = w[dx == 0 ? HB + 2 : (dx == 1 ? 0 : 1)];
-      } else {
-        v = w[1 - dx];
-      }
-      return v;
+      return w[1 - dx];
     }
   };
 
   // collide plane c = zb + k: the laterally moving populations go to the window, the
   // others to their destinations (rest: plane c, -z: c - 1, +z: c + 1)
-  auto produce = [&](int k, R* win, V& rest, V& down, V& up) {
+  auto produce = [&](int k, R* win, R& rest, R& down, R& up) {
     slot_wait(k);
     if (active) {
-      const R* sl = slots + (k % NS) * SLOTN + NPT * tid;
-      Coef<V> kc;
-      each_coef<L, V>(kc, [&](auto I, V& v) { v = *reinterpret_cast<const V*>(sl + decltype(I)::value * (BX * BY)); });
-      rest = post_v<L, 0>(kc);
+      const R* sl = slots + (k % NS) * SLOTN + tid;
+      Coef<R> kc;
+      each_coef<L, R>(kc, [&](auto I, R& v) { v = sl[decltype(I)::value * (BX * BY)]; });
+      rest = post<L, R, 0>(kc);
       static_for<1, Q>([&](auto A_) {
         constexpr int a = decltype(A_)::value;
         constexpr int b = L::opp(a);
         if constexpr (leading_sign<L>(a) == 1) {
-          V fa, fb;
+          R fa, fb;
           post_pair<L, a>(kc, fa, fb);
           if constexpr (is_lateral<L>(a)) {
             put(win, A_, fa);
@@ -513,7 +450,7 @@ __device__ __forceinline__ void k3_brick(
 
   // gathered populations of three destination planes; the roles of the sets
   // are permuted at compile time
-  V G[3][Q];
+  R G[3][Q];
   produce(0, win0, G[1][0], G[0][zm], G[2][zp]);
   window_ready(0);
   window_wait(0);
@@ -523,14 +460,14 @@ __device__ __forceinline__ void k3_brick(
     constexpr int k = decltype(K)::value;
     const int g = zb + 3 * t + k;
     const int kc = 3 * t + k + 1;  // plane c's index
-    V(&G0)[Q] = G[k % 3];          // destination plane g - 1
-    V(&G1)[Q] = G[(k + 1) % 3];    // g
-    V(&G2)[Q] = G[(k + 2) % 3];    // g + 1
+    R(&G0)[Q] = G[k % 3];          // destination plane g - 1
+    R(&G1)[Q] = G[(k + 1) % 3];    // g
+    R(&G2)[Q] = G[(k + 2) % 3];    // g + 1
     const int c = g + 1;
     const R* win_g = win0 + (kc - 1) % NW * WSTRIDE;
     R* win_c = win0 + kc % NW * WSTRIDE;
-    V up_c = V(R(0));  // plane c's +z population: of plane c + 1, whose set is G0
-    const V down_g = G0[zm], up_g = G2[zp];  // this node's own, for a z wall's bounce-back
+    R up_c = R(0);  // plane c's +z population: of plane c + 1, whose set is G0
+    const R down_g = G0[zm], up_g = G2[zp];  // this node's own, for a z wall's bounce-back
     if (c <= ze) {
       produce(kc, win_c, G2[0], G1[zm], up_c);
       window_ready(kc);
@@ -542,7 +479,7 @@ __device__ __forceinline__ void k3_brick(
           constexpr int a = decltype(A_)::value;
           constexpr int cx = L::cx(a), cy = L::cy(a), cz = L::cz(a);
           if constexpr (is_lateral<L>(a)) {
-            const V v = get(win_g, A_, std::integral_constant<int, cx>{}, std::integral_constant<int, cy>{});
+            const R v = get(win_g, A_, std::integral_constant<int, cx>{}, std::integral_constant<int, cy>{});
             if constexpr (cz == -1) G0[a] = v;
             if constexpr (cz == 0) G1[a] = v;
             if constexpr (cz == 1) G2[a] = v;
@@ -557,7 +494,7 @@ __device__ __forceinline__ void k3_brick(
             if constexpr (cz != 0) {
               if (cz == 1 ? z_lo : z_hi) {
                 constexpr int oa = L::opp(a);
-                V v;
+                R v;
                 if constexpr (is_lateral<L>(oa))
                   v = get(win_g, std::integral_constant<int, oa>{}, std::integral_constant<int, 0>{},
                           std::integral_constant<int, 0>{});
@@ -566,14 +503,9 @@ __device__ __forceinline__ void k3_brick(
                 int cb = 4;
                 if constexpr (cy == 1) cb |= y == 0 && !args.per[1] ? 2 : 0;
                 if constexpr (cy == -1) cb |= y == ny - 1 && !args.per[1] ? 2 : 0;
-#pragma unroll
-                for (int l = 0; l < NPT; ++l) {
-                  int cl = cb;
-                  if constexpr (cx == 1) cl |= x + l == 0 && !args.per[0] ? 1 : 0;
-                  if constexpr (cx == -1) cl |= x + l == nx - 1 && !args.per[0] ? 1 : 0;
-                  lane_of(v, l) = lane_of(v, l) + args.bb[a][cl];
-                }
-                G1[a] = v;
+                if constexpr (cx == 1) cb |= x == 0 && !args.per[0] ? 1 : 0;
+                if constexpr (cx == -1) cb |= x == nx - 1 && !args.per[0] ? 1 : 0;
+                G1[a] = v + args.bb[a][cb];
               }
             }
           });
@@ -583,36 +515,29 @@ __device__ __forceinline__ void k3_brick(
       const int zd = g - 1;
       if (zd >= z0) {
         if constexpr (POP) {
-          static_assert(NPT == 1, "one node per thread");
           S* o = static_cast<S*>(args.pop) + (x + args.pitch * y + plane * zd);
           static_for<0, Q>([&](auto A_) {
             constexpr int a = decltype(A_)::value;
             o[a * args.vol] = store_as<S, R>(G0[a]);
           });
         } else {
-          V fr[Q];
+          R fr[Q];
           static_for<0, Q>([&](auto A_) {
             constexpr int a = decltype(A_)::value;
-            fr[a] = round_value<S>(G0[a]);
+            fr[a] = round_to_storage<S, R>(G0[a]);
           });
-          Coef<V> kc2;
+          Coef<R> kc2;
           moments_coeffs<L, FORCE>(fr, args.ph, kc2);
           char* o = reinterpret_cast<char*>(out0 + plane * zd);
           const uint32_t v32 = args.vol32;
-          if (NPT == 1 || act1) {
-            each_coef<L, V>(kc2, [&](auto I, V& v) {
-              *reinterpret_cast<V*>(o + uint64_t(v32) * uint32_t(decltype(I)::value * 32 * sizeof(R))) = v;
-            });
-          } else {
-            each_coef<L, V>(kc2, [&](auto I, V& v) {
-              *reinterpret_cast<R*>(o + uint64_t(v32) * uint32_t(decltype(I)::value * 32 * sizeof(R))) = lane_of(v, 0);
-            });
-          }
+          each_coef<L, R>(kc2, [&](auto I, R& v) {
+            *reinterpret_cast<R*>(o + uint64_t(v32) * uint32_t(decltype(I)::value * 32 * sizeof(R))) = v;
+          });
           if (west || east) {
             R* e = edge0 + int64_t(ny) * NC * zd;
-            put_record<L>(kc2, e, west ? 0 : eastl);
-            // a tile of one column pair is both
-            if (west && east) put_record<L>(kc2, e + int64_t(args.ntx) * ny * nz * NC, eastl);
+            put_record<L>(kc2, e);
+            // a tile of one column is both
+            if (west && east) put_record<L>(kc2, e + int64_t(args.ntx) * ny * nz * NC);
           }
         }
       }
@@ -649,13 +574,12 @@ __device__ __forceinline__ void k3_brick(
   }
 }
 
-template <class L, class S, class R, int BX, int BY, int NS, int NPT, bool FORCE, int MINB, bool POP = false>
-__global__ void __launch_bounds__(K3Shape<L, R, BX, BY, NS, NPT, MINB>::NT, MINB)
-    k3_step(const __grid_constant__ CUtensorMap tmap,
-            const __grid_constant__ K3Args<R, typename K3Shape<L, R, BX, BY, NS, NPT, MINB>::V> args) {
+template <class L, class S, class R, int BX, int BY, int NS, bool FORCE, int MINB, bool POP = false>
+__global__ void __launch_bounds__(K3Shape<L, R, BX, BY, NS, MINB>::NT, MINB)
+    k3_step(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ K3Args<R> args) {
   const int b = blockIdx.x;
-  k3_brick<L, S, R, BX, BY, NS, NPT, FORCE, MINB, POP>(&tmap, args, b % args.ntx, (b / args.ntx) % args.nty,
-                                                       b / (args.ntx * args.nty));
+  k3_brick<L, S, R, BX, BY, NS, FORCE, MINB, POP>(&tmap, args, b % args.ntx, (b / args.ntx) % args.nty,
+                                                  b / (args.ntx * args.nty));
 }
 
 // Populations -> coefficient fields and edge records, node by node (each thread
@@ -679,8 +603,8 @@ __global__ void __launch_bounds__(256)
     each_coef<L, R>(kc, [&](auto I, R& v) { dst[decltype(I)::value * vol + i] = v; });
     const int tI = x / bx, xl = x - tI * bx, ntx = (nx + bx - 1) / bx;
     constexpr int NC = n_coef<L>();
-    if (xl == 0) put_record<L>(kc, edst + k3_edge(0, tI, ntx, rows, row) * NC, 0);
-    if (xl == bx - 1 || x == nx - 1) put_record<L>(kc, edst + k3_edge(1, tI, ntx, rows, row) * NC, 0);
+    if (xl == 0) put_record<L>(kc, edst + k3_edge(0, tI, ntx, rows, row) * NC);
+    if (xl == bx - 1 || x == nx - 1) put_record<L>(kc, edst + k3_edge(1, tI, ntx, rows, row) * NC);
   }
 }
 

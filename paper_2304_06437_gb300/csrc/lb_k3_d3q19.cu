@@ -1,6 +1,6 @@
 // lb_k3_d3q19.cu -- compiled tiles of the step in moment form for D3Q19.
-// Each entry: storage / arithmetic type, tile bx x by, TMA ring depth, nodes
-// per thread, CTAs per SM; and the brick cross-sections whose contexts can end a
+// Each entry: storage / arithmetic type, tile bx x by, TMA ring depth, CTAs
+// per SM; and the brick cross-sections whose contexts can end a
 // run: all that are compiled, so that no batch, autotuner or requested brick takes a
 // context's runs away.
 #include "lb_k3_launch.cuh"
@@ -8,11 +8,11 @@
 namespace lbgb {
 
 extern const K3Variant k3_variants_d3q19[] = {
-    K3Impl<D3Q19, float, float, 32, 16, 3, 1, 1>::variant(LB_D3Q19, LB_F32),
-    K3Impl<D3Q19, float, float, 32, 4, 2, 1, 2>::variant(LB_D3Q19, LB_F32),  // small domains
-    K3Impl<D3Q19, double, double, 32, 8, 2, 1, 1>::variant(LB_D3Q19, LB_F64),
-    K3Impl<D3Q19, __half, float, 32, 16, 3, 1, 1>::variant(LB_D3Q19, LB_F16S),
-    K3Impl<D3Q19, __nv_bfloat16, float, 32, 16, 3, 1, 1>::variant(LB_D3Q19, LB_BF16S),
+    K3Impl<D3Q19, float, float, 32, 16, 3, 1>::variant(LB_D3Q19, LB_F32),
+    K3Impl<D3Q19, float, float, 32, 4, 2, 2>::variant(LB_D3Q19, LB_F32),  // small domains
+    K3Impl<D3Q19, double, double, 32, 8, 2, 1>::variant(LB_D3Q19, LB_F64),
+    K3Impl<D3Q19, __half, float, 32, 16, 3, 1>::variant(LB_D3Q19, LB_F16S),
+    K3Impl<D3Q19, __nv_bfloat16, float, 32, 16, 3, 1>::variant(LB_D3Q19, LB_BF16S),
 };
 extern const int k3_n_variants_d3q19 = sizeof(k3_variants_d3q19) / sizeof(k3_variants_d3q19[0]);
 

@@ -11,7 +11,7 @@ namespace lbgb {
 
 // A compiled tile of k3_step (lattice x storage x bx x by).
 struct K3Variant {
-  int lattice, storage, bx, by, ns, npt, minb;
+  int lattice, storage, bx, by, ns, minb;
   cudaError_t (*configure)();
   // one step of the context's domain: set src (0 = A, 1 = B) to the other
   cudaError_t (*step)(lb_ctx*, int src);
@@ -32,21 +32,20 @@ struct LeaveVariant {
   cudaError_t (*leave)(lb_ctx*);
 };
 
-template <class L, class S, class R, int BX, int BY, int NS, int NPT, int MINB>
+template <class L, class S, class R, int BX, int BY, int NS, int MINB>
 struct K3Impl {
-  using Sh = K3Shape<L, R, BX, BY, NS, NPT, MINB>;
-  using V = typename Sh::V;
+  using Sh = K3Shape<L, R, BX, BY, NS, MINB>;
   static constexpr bool HALF = sizeof(S) == 2;
 
   static cudaError_t configure() {
-    cudaError_t e = cudaFuncSetAttribute(k3_step<L, S, R, BX, BY, NS, NPT, false, MINB>,
+    cudaError_t e = cudaFuncSetAttribute(k3_step<L, S, R, BX, BY, NS, false, MINB>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, int(Sh::SMEM));
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k3_step<L, S, R, BX, BY, NS, NPT, true, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      e = cudaFuncSetAttribute(k3_step<L, S, R, BX, BY, NS, true, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                int(Sh::SMEM));
     if constexpr (HALF)
       if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k3_step<L, S, R, BX, BY, NS, NPT, false, MINB, true>,
+        e = cudaFuncSetAttribute(k3_step<L, S, R, BX, BY, NS, false, MINB, true>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, int(Sh::SMEM));
     return e;
   }
@@ -60,10 +59,10 @@ struct K3Impl {
     return static_cast<R*>(ctx->f) + moment_edge_at(ctx->g, ctx->storage) + which * moment_edge_elems(ctx->g, BX);
   }
 
-  static K3Args<R, V> args_of(lb_ctx* ctx, int src) {
+  static K3Args<R> args_of(lb_ctx* ctx, int src) {
     const Geometry& g = ctx->g;
-    K3Args<R, V> a;
-    a.ph = make_phys<V>(g);
+    K3Args<R> a;
+    a.ph = make_phys<R>(g);
     a.nx = g.nx;
     a.ny = g.ny;
     a.nz = g.nz;
@@ -88,20 +87,20 @@ struct K3Impl {
   }
 
   static cudaError_t step(lb_ctx* ctx, int src) {
-    const K3Args<R, V> a = args_of(ctx, src);
+    const K3Args<R> a = args_of(ctx, src);
     const int grid = a.ntx * a.nty * a.ntz;
     const CUtensorMap& tm = ctx->mr.maps[src];
     const bool early = !ctx->mr.shared && grid <= k1_sm_count() * MINB;
-    return launch_step(ctx->g.has_force ? k3_step<L, S, R, BX, BY, NS, NPT, true, MINB>
-                                        : k3_step<L, S, R, BX, BY, NS, NPT, false, MINB>,
+    return launch_step(ctx->g.has_force ? k3_step<L, S, R, BX, BY, NS, true, MINB>
+                                        : k3_step<L, S, R, BX, BY, NS, false, MINB>,
                        grid, Sh::NT, Sh::SMEM, ctx->stream, early, tm, a);
   }
 
   // (no collision: one instantiation serves with and without a force)
   static cudaError_t leave(lb_ctx* ctx) {
     if constexpr (HALF) {
-      const K3Args<R, V> a = args_of(ctx, 0);
-      k3_step<L, S, R, BX, BY, NS, NPT, false, MINB, true>
+      const K3Args<R> a = args_of(ctx, 0);
+      k3_step<L, S, R, BX, BY, NS, false, MINB, true>
           <<<a.ntx * a.nty * a.ntz, Sh::NT, Sh::SMEM, ctx->stream>>>(ctx->mr.maps[0], a);
     }
     return cudaGetLastError();
@@ -122,7 +121,7 @@ struct K3Impl {
   }
 
   static constexpr K3Variant variant(int lattice, int storage) {
-    return K3Variant{lattice, storage, BX, BY, NS, NPT, MINB, &configure, &step, &enter, HALF ? &leave : nullptr};
+    return K3Variant{lattice, storage, BX, BY, NS, MINB, &configure, &step, &enter, HALF ? &leave : nullptr};
   }
 };
 

@@ -31,7 +31,6 @@
 #include <cmath>
 
 #include "lb_k1_launch.cuh"
-#include "lb_pair.cuh"
 
 namespace lbgb {
 namespace {
