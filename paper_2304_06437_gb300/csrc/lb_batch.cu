@@ -509,7 +509,8 @@ int lb_batch_step(lb_batch* b, int64_t n) {
   int rc = LB_OK;
   if (n >= kMomentMinSteps && !b->runs.empty()) {
     LB_BTRY(cudaEventRecord(b->done, b->stream));
-    for (cudaStream_t st : b->lanes) LB_BTRY(cudaStreamWaitEvent(st, b->done, 0));
+    for (cudaStream_t st : b->lanes)
+      if (rc == LB_OK) rc = cuda_rc(cudaStreamWaitEvent(st, b->done, 0));
     for (size_t k = 0; k < b->runs.size() && rc == LB_OK; ++k) {
       lb_ctx* x = b->ctxs[b->runs[k]];
       // the launches of a run go to the stream of the context
@@ -517,22 +518,27 @@ int lb_batch_step(lb_batch* b, int64_t n) {
       x->stream = b->lanes[b->lane[k]];
       rc = cuda_rc(x->g.d == 3 ? moment_run_beside(x, n) : flat_run(x, n, true));
       x->stream = own;
-      x->steps_done += n;
     }
     if (rc == LB_OK && !b->rest.empty()) rc = step_classes(*b, b->rest, b->rest_graph, n);
+    // the batch stream waits for what the lanes were given, also where a later
+    // launch failed: nothing may run behind the caller's back
     for (size_t k = 0; k < b->lanes.size(); ++k) {
-      LB_BTRY(cudaEventRecord(b->lane_ev[k], b->lanes[k]));
-      LB_BTRY(cudaStreamWaitEvent(b->stream, b->lane_ev[k], 0));
+      cudaError_t e = cudaEventRecord(b->lane_ev[k], b->lanes[k]);
+      if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, b->lane_ev[k], 0);
+      if (rc == LB_OK) rc = cuda_rc(e);
     }
+    if (rc == LB_OK)
+      for (int i : b->runs) b->ctxs[i]->steps_done += n;
   } else {
     rc = step_classes(*b, b->classes, b->graph, n);
   }
-  if (rc != LB_OK) return rc;
-  b->steps_done += n;
   // later work on a member's stream sees the batch's steps
-  LB_BTRY(cudaEventRecord(b->done, b->stream));
-  for (lb_ctx* x : b->ctxs) LB_BTRY(cudaStreamWaitEvent(x->stream, b->done, 0));
-  return LB_OK;
+  cudaError_t e = cudaEventRecord(b->done, b->stream);
+  for (lb_ctx* x : b->ctxs)
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(x->stream, b->done, 0);
+  if (rc == LB_OK) rc = cuda_rc(e);
+  if (rc == LB_OK) b->steps_done += n;
+  return rc;
 }
 
 int lb_batch_sync(lb_batch* b) {
@@ -611,6 +617,7 @@ void lb_batch_destroy(lb_batch* b) {
   if (!b) return;
   DevGuard guard(b->device);
   if (b->stream) cudaStreamSynchronize(b->stream);
+  for (cudaStream_t st : b->lanes) cudaStreamSynchronize(st);
   if (b->graph) cudaGraphExecDestroy(b->graph);
   if (b->rest_graph) cudaGraphExecDestroy(b->rest_graph);
   for (auto& c : b->classes) free_class(c);
