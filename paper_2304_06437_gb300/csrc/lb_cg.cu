@@ -693,7 +693,7 @@ int lb_cg_step(lb_cg* c, int64_t n) {
                                 reinterpret_cast<R*>(fb) + 4 * N}};
       const int grid = int(c->g.ntx * c->g.nty * c->g.ntz);
       // about one wave of the step's blocks (128 x 96 D2Q9 FP32: 10.7 -> 5.7 us a step)
-      const bool early = grid <= 4 * 152;
+      const bool early = grid <= 4 * k1_sm_count();
       auto gradient = [&](int which, auto pull) {
         constexpr bool P = decltype(pull)::value;
         launch_step(c->nci_amp != 0.0 ? cg_gradient_kernel<L, S, R, true, P> : cg_gradient_kernel<L, S, R, false, false>,

@@ -129,6 +129,7 @@ void drop_step_graph(lb_ctx* ctx);
 cudaError_t k1_step(lb_ctx* ctx);
 cudaError_t k1_bootstrap(lb_ctx* ctx);  // fill the current shell parity from f
 cudaError_t k1_configure(lb_ctx* ctx);  // one-time kernel attributes
+int k1_sm_count();  // of the current device (152 where none is visible)
 
 // ---- runs of several steps in moment form (lb_k3_plan.cu)
 // arithmetic-type elements that the two coefficient sets and their edge

@@ -38,7 +38,6 @@ struct K1Variant {
 
 // the compiled shape a fused-scheme context runs (lb_k1_plan.cu)
 const K1Variant* k1_ctx_variant(lb_ctx* ctx);
-int k1_sm_count();
 
 // blocks of eight warps for k1_bootstrap's items: rows in pieces of about 256
 // columns, one to a warp
