@@ -499,6 +499,18 @@ def fused_plan(lattice, dims, storage="f32", tile=None, sms=0) -> dict:
     return {name: getattr(p, name) for name, _ in p._fields_}
 
 
+def flat_plan(dims, n, storage="f32", sms=0) -> dict:
+    """How a run of n steps of a 2D domain is divided into launches
+    (lb_plan_flat; no device is touched)."""
+    lib = B.load()
+    st = B.STORAGES[storage] if isinstance(storage, str) else int(storage)
+    dims = (list(dims) + [1, 1])[:3]
+    p = B.lb_flat_plan_t()
+    B.check(lib.lb_plan_flat(st, (ctypes.c_int64 * 3)(*[int(v) for v in dims]), int(n), int(sms), ctypes.byref(p)),
+            "lb_plan_flat")
+    return {name: getattr(p, name) for name, _ in p._fields_}
+
+
 def context_bytes(lattice, dims, storage="f32") -> dict:
     """Device memory that a fused context may take (lb_plan_memory; no device
     is touched)."""
