@@ -122,7 +122,8 @@ typedef struct {
 LB_API void lb_default_options(lb_options* opt);
 
 /* Creates a context: allocates the population array (and the shell or moment
- * buffers of the chosen scheme) on the device and zeroes the state (rest at
+ * buffers of the chosen scheme, and memory for runs of several steps:
+ * lb_plan_memory()) on the device and zeroes the state (rest at
  * rho0).  dims[2] must be 1 for D2Q9.  tau > 1/2 (nu = (tau - 1/2)/3, section
  * 2).  bnd may be NULL (all periodic); opt may be NULL (defaults).
  * Errors: LB_E_INVAL for bad sizes/kinds, LB_E_NOMEM, LB_E_CUDA. */
@@ -155,13 +156,19 @@ LB_API int lb_get_region(lb_ctx* ctx, const int64_t lo[3], const int64_t size[3]
 /* Enqueues n time steps on the context stream (asynchronous).  Each step is
  * one application of the step of section 3 (Eq. LBexp with fhat^neq, the
  * multline step equation) with the walls of section 5.1.  For n >= 4 the
- * fused scheme launches a pair of steps captured once as a CUDA graph (held
- * by the context until it is re-planned or destroyed); if the caller is
- * capturing the context stream, the steps are launched one by one and land
- * in the caller's graph, which can be replayed where it holds an even number of
+ * fused scheme takes the steps of one call as a run: between them a node's state
+ * is its post-collision coefficients (6 in 2D, 10 in 3D) instead of its
+ * populations, on tiles of the library's choice whatever the context's brick,
+ * and 2D runs take several steps per launch.  The populations at its end are
+ * those of n calls of one step, bit for bit.  A run needs the memory that
+ * lb_plan_memory() names; a context that did not get it, and 2D domains in
+ * 16-bit storage, launch a pair of steps captured once as a CUDA graph instead.
+ * Recorded launches are held by the context until it is re-planned or destroyed.
+ * If the caller is capturing the context stream, all launches land in the
+ * caller's graph, which can be replayed where it holds an even number of
  * steps, also between other calls, as long as those took an even number of
- * steps in all since the capture.  Errors: LB_E_INVAL (n < 0, or n > 1 on a slab with
- * a link face), LB_E_CUDA (a launch failed). */
+ * steps in all since the capture.  Errors: LB_E_INVAL (n < 0, or n > 1 on a
+ * slab with a link face), LB_E_CUDA (a launch failed). */
 LB_API int lb_step(lb_ctx* ctx, int64_t n);
 
 /* Density rho [N] and velocity u [d][N] of the stored state, FP64 results.
@@ -211,8 +218,8 @@ LB_API int lb_lattice_table(int32_t lattice, int32_t* c, double* w, int32_t* opp
  * full-size arrays and bytes per node each schedule keeps for a lattice --
  * the paper's moment scheme (q + m arrays), a two-array "flip-flop" scheme
  * (2q + d + 1 arrays) and this library's fused single-array scheme (q arrays
- * plus the shell, reported separately by lb_info).  s = bytes per value.
- * Needs no GPU. */
+ * plus the shell and the memory of runs, reported separately by lb_info).
+ * s = bytes per value.  Needs no GPU. */
 typedef struct {
   int32_t q, m;                 /* populations, stored moments 1 + d + d(d+1)/2 */
   int32_t arrays_moment_scheme; /* q + m      (15 for D2Q9, 29 for D3Q19) */
@@ -346,8 +353,9 @@ LB_API int lb_autotune(lb_ctx* ctx, int32_t steps, lb_tune_entry* table, int32_t
  * bricks per persistent CTA, its members' sweeps are halved (down to 64
  * planes) until it has.  Classes run on parallel branches of the graph.
  * Calls of four or more steps take the largest members, as many as have 160 Ki
- * nodes (2D: 64 Ki) on average, through the runs that lb_step() has for several steps, on
- * streams of the batch and beside the classes of the other members.
+ * nodes (2D: 64 Ki) on average, through the runs that lb_step() has for several
+ * steps, on streams of the batch and beside the classes of the other members
+ * (lb_batch_alone() names them).
  * stream: cudaStream_t for the batch's work, NULL = a library-owned stream.
  * Errors: LB_E_INVAL (NULL, duplicates, mixed devices), LB_E_UNSUPPORTED,
  * LB_E_NOMEM, LB_E_CUDA. */
